@@ -88,7 +88,7 @@ typedef struct {
  *   opt    NULL for defaults.
  *   stream used for the layout check; create synchronizes this stream.
  * Allocates scratch and output buffers sized from V, T and H (about
- * 8 bytes per triangle of scratch plus 4*(T + T+1 + 3T + 3T) bytes of
+ * 20 bytes per triangle of scratch plus 4*(T + T+1 + 3T + 3T) bytes of
  * output); polylla_generate then allocates and frees nothing (the paper's
  * point in Section 4.2: the method runs in the input's own memory).
  * Errors: INVALID_ARGUMENT, INVALID_MESH (twin not an involution without
@@ -543,7 +543,7 @@ void polylla_server_destroy(polylla_server *srv);
  * runs the same kernels as polylla_generate, but their scratch (labels, tip
  * lists, output tile words, counters) lives in one static device array of
  * fixed size that every GPU loading the library holds until the process
- * exits (about 1.7 MB), so no context, no cudaMalloc and no cudaFree.
+ * exits (about 3.2 MB), so no context, no cudaMalloc and no cudaFree.
  *
  *   mesh    device arrays as for polylla_create; must satisfy the layout
  *           polylla_create checks (no check is made here);

@@ -221,10 +221,14 @@ static int alloc_work(polylla_ctx *c, const polylla_options *opt) {
     c->w.group_tot = (unsigned long long *)p;
     if ((rc = dev_alloc(c, &p, sizeof(unsigned long long) * (size_t)(c->w.n_tile_max / SCAN_THREADS + 1)))) return rc;
     c->w.group_pre = (unsigned long long *)p;
-    if ((rc = dev_alloc(c, &p, sizeof(unsigned long long) * (size_t)out_rec_count(T)))) return rc;
-    c->w.poly_rec = (unsigned long long *)p;
+    if ((rc = dev_alloc(c, &p, sizeof(uint32_t) * (size_t)T))) return rc;
+    c->w.poly_rec = (uint32_t *)p;
     if ((rc = dev_alloc(c, &p, sizeof(unsigned long long) * (size_t)out_warp_count(T)))) return rc;
     c->w.poly_wtot = (unsigned long long *)p;
+    c->w.cross_own = (int32_t)cross_own_count(T);
+    c->w.cross_more = (int32_t)cross_more_count(T);
+    if ((rc = dev_alloc(c, &p, 64 * (size_t)(cross_own_count(T) + cross_more_count(T))))) return rc;
+    c->w.cross_pool = (int32_t *)p;
     if ((rc = dev_alloc(c, &p, sizeof(int32_t) * (size_t)T))) return rc;
     c->w.seeds = (int32_t *)p;
     if ((rc = dev_alloc(c, &p, sizeof(int32_t) * (size_t)(T + 1)))) return rc;
@@ -873,11 +877,9 @@ int polylla_convexify(polylla_ctx *c, polylla_stream stream) {
         c->cv_cap = 3 * c->mesh.T;
     }
     c->last_stream = s;
-    const int32_t tile = polygons_config_valid(c->w.out_tile, c->w.out_items) ? c->w.out_tile : OUT_TILE_DEFAULT;
-    const size_t n_tiles = ((size_t)c->mesh.T + tile - 1) / tile;
     CK(cudaMemsetAsync(c->cv_count, 0, 2 * sizeof(int32_t), s));
-    CK(cudaMemsetAsync(c->w.tile_state, 0, sizeof(unsigned long long) * n_tiles, s));
-    CK(cudaMemsetAsync(&c->w.ctrl->scan_done, 0, sizeof(int32_t), s));
+    CK(cudaMemsetAsync(c->w.tile_state, 0, sizeof(unsigned long long) * (size_t)c->w.n_tile_max, s));
+    CK(cudaMemsetAsync(&c->w.ctrl->scan_done, 0, 2 * sizeof(int32_t), s));  // and cross_used
     launch_convex_chords(c->mesh, c->w, c->cv_reflex, c->cv_count + 1, c->cv_list, c->cv_count, c->cv_cap, s);
     launch_convex_mark(c->mesh, c->w, c->cv_list, c->cv_count, c->cv_cap, s);
     launch_chord_links_list(c->mesh, c->w, c->cv_list, c->cv_count, c->cv_cap, s);

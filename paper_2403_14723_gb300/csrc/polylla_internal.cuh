@@ -12,9 +12,12 @@
 //                        tile, and their exclusive scan within groups of
 //                        1024 tiles; group_tot, group_pre [T/2^20 + 1] u64 the
 //                        groups' totals and their exclusive scan
-//   poly_rec [T/2+2049] u64  per output thread: its (polygons, length)
-//                        offset in its warp's range and the mask of its minima
-//   poly_wtot [T/128+34] u64  per output warp: its (polygons, length) total
+//   poly_rec [T] u32     per polygon, at its output warp's first triangle on:
+//                        its minimum within the warp's half-edges, its length
+//                        and its chunk of the pool
+//   cross_pool [T/8+T/32+512][16] i32  the half-edges that a polygon which
+//                        leaves its tile visits from there on
+//   poly_wtot [T/64+66] u64  per output warp: its (polygons, length) total
 //   seeds [T], offsets [T+1], he_list [3T], v_list [3T]   CSR output
 //   ctrl          DevCtrl       counters and the device error word
 // A batch context adds the union origin/twin/next/prev [H] (origin and the
@@ -42,7 +45,8 @@ struct DevCtrl {
     int32_t n_polygons;   // P
     int32_t n_frontier;   // N_F
     int32_t scan_done;    // tile-scan blocks finished
-    int32_t pad[3];
+    int32_t cross_used;   // chunks asked for from the common part of the crossing walks' pool
+    int32_t pad[2];
 };
 
 struct MeshView {
@@ -61,11 +65,14 @@ struct Work {
     int32_t *chords;
     int32_t tip_cap;
     unsigned long long *tile_state; // (polygons, length) total per output tile [n_tile_max]
-    unsigned long long *tile_pre;   // their exclusive scan within groups of SCAN_THREADS tiles
+    unsigned long long *tile_pre;   // the totals' exclusive scan within groups of SCAN_THREADS tiles
     unsigned long long *group_tot;  // each group's total [n_tile_max / SCAN_THREADS + 1]
     unsigned long long *group_pre;  // their exclusive scan [n_tile_max / SCAN_THREADS + 1]
-    unsigned long long *poly_rec;   // per output thread: its place in its warp and its minima [n_rec_max]
+    uint32_t *poly_rec;             // per polygon: its minimum within its warp's half-edges, its length [T]
     unsigned long long *poly_wtot;  // per output warp: (polygons, length) of its range
+    int32_t *cross_pool;            // chunks of 16 words: crossing walks' half-edges from their tile on
+    int32_t cross_own;              // the tiles' own chunks, at the start of cross_pool
+    int32_t cross_more;             // chunks after them, for the walks that need more than one
     int32_t n_tile_max;             // ceil(T / OUT_TILE_MIN)
     int32_t out_tile;               // output tile: triangles
     int32_t out_items;              // output kernel: triangles per thread
@@ -121,11 +128,18 @@ struct BatchView {
 constexpr int OUT_TILE_MIN = 1024;
 constexpr int OUT_TILE_MAX = 4096;
 constexpr int OUT_ITEMS_MIN = 2;
-constexpr int OUT_TILE_DEFAULT = 2048;
+constexpr int OUT_TILE_DEFAULT = 1024;
 constexpr int OUT_ITEMS_DEFAULT = 4;
-// per-thread records of the output stage for T triangles, any configuration
-__host__ __device__ constexpr int64_t out_rec_count(int64_t T) { return (T + OUT_TILE_MAX) / OUT_ITEMS_MIN + 1; }
-__host__ __device__ constexpr int64_t out_warp_count(int64_t T) { return out_rec_count(T) / 32 + 2; }
+// output warps (of 32 triangles per thread at least OUT_ITEMS_MIN) for T
+// triangles, any configuration
+__host__ __device__ constexpr int64_t out_warp_count(int64_t T) { return (T + OUT_TILE_MAX) / (32 * OUT_ITEMS_MIN) + 2; }
+// chunks of the crossing walks' pool: one per XQUOTA triangles for the tile
+// that holds them (0.06 polygons per triangle leave a tile of 1,024 on
+// grids, 0.02 on Delaunay meshes; the walks that find no chunk cost the
+// listing kernel a chain of loads), then those for long walks
+constexpr int XQUOTA = 8;
+__host__ __device__ constexpr int64_t cross_own_count(int64_t T) { return (T + OUT_TILE_MAX) / XQUOTA; }
+__host__ __device__ constexpr int64_t cross_more_count(int64_t T) { return T / 32 + 256; }
 constexpr int SCAN_THREADS = 1024;
 
 // longest-edge kernel: persistent warps, each with a two-stage ring of

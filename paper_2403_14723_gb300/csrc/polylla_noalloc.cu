@@ -35,8 +35,9 @@ constexpr size_t OFF_TILE_PRE = OFF_TILES + up256(8 * (size_t)NA_MAX_TILES);
 constexpr size_t OFF_GROUPS = OFF_TILE_PRE + up256(8 * (size_t)NA_MAX_TILES);
 constexpr size_t OFF_GROUP_PRE = OFF_GROUPS + up256(8 * (size_t)(NA_MAX_TILES / SCAN_THREADS + 1));
 constexpr size_t OFF_REC = OFF_GROUP_PRE + up256(8 * (size_t)(NA_MAX_TILES / SCAN_THREADS + 1));
-constexpr size_t OFF_WTOT = OFF_REC + up256(8 * (size_t)out_rec_count(NA_MAX_T));
-constexpr size_t OFF_CTRL = OFF_WTOT + up256(8 * (size_t)out_warp_count(NA_MAX_T));
+constexpr size_t OFF_WTOT = OFF_REC + up256(4 * (size_t)NA_MAX_T);
+constexpr size_t OFF_POOL = OFF_WTOT + up256(8 * (size_t)out_warp_count(NA_MAX_T));
+constexpr size_t OFF_CTRL = OFF_POOL + up256(64 * (size_t)(cross_own_count(NA_MAX_T) + cross_more_count(NA_MAX_T)));
 constexpr size_t NA_BYTES = OFF_CTRL + up256(sizeof(DevCtrl));
 
 constexpr int kMaxDevices = 64;
@@ -44,7 +45,7 @@ constexpr int kMaxDevices = 64;
 }  // namespace
 
 // The scratch.  Every GPU that loads the library holds it (NA_BYTES, about
-// 1.7 MB) until the process exits.  In host code its name is only a host-side
+// 3.2 MB) until the process exits.  In host code its name is only a host-side
 // stand-in: the device address comes from cudaGetSymbolAddress below.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_BYTES];
 
@@ -114,8 +115,11 @@ extern "C" int polylla_generate_noalloc(const polylla_mesh *mesh, int32_t *seeds
     w.tile_pre = reinterpret_cast<unsigned long long *>(base + OFF_TILE_PRE);
     w.group_tot = reinterpret_cast<unsigned long long *>(base + OFF_GROUPS);
     w.group_pre = reinterpret_cast<unsigned long long *>(base + OFF_GROUP_PRE);
-    w.poly_rec = reinterpret_cast<unsigned long long *>(base + OFF_REC);
+    w.poly_rec = reinterpret_cast<uint32_t *>(base + OFF_REC);
     w.poly_wtot = reinterpret_cast<unsigned long long *>(base + OFF_WTOT);
+    w.cross_pool = reinterpret_cast<int32_t *>(base + OFF_POOL);
+    w.cross_own = (int32_t)cross_own_count(NA_MAX_T);
+    w.cross_more = (int32_t)cross_more_count(NA_MAX_T);
     w.n_tile_max = (int32_t)(((int64_t)T + OUT_TILE_MIN - 1) / OUT_TILE_MIN);
     w.seeds = seeds;
     w.offsets = offsets;
