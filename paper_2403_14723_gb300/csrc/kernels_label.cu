@@ -428,6 +428,20 @@ void launch_longest_edge(const MeshView &m, const Work &w, cudaStream_t s) {
 // ===========================================================================
 __device__ __forceinline__ int32_t div3(int32_t x) { return (int32_t)((uint32_t)x / 3u); }
 
+// A rotation came back to its tip's only frontier half-edge f, steps steps past
+// CW^2(f): the tip has degree steps + 2, which k_chords reads in the chord's
+// place (choosing the chord here, by walking half of the rotation again, made
+// the relink of Delaunay meshes 5 % slower: a tip in every fourth warp).
+__device__ __forceinline__ void add_tip(const Work &w, int32_t f, int32_t steps) {
+    const int32_t sl = atomicAdd(&w.ctrl->n_tips, 1);
+    if (sl < w.tip_cap) {
+        w.tips[sl] = f;
+        w.chords[sl] = steps + 2;
+    } else {
+        atomicOr(&w.ctrl->error, DEV_ERR_CAPACITY);
+    }
+}
+
 template <int NT, int IPT, bool BATCH>
 __global__ void __launch_bounds__(NT, 2048 / NT / IPT) k_label_relink(MeshView m, Work w) {
     constexpr int TT = NT * IPT;  // triangles per CTA
@@ -546,11 +560,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT / IPT) k_label_relink(MeshView m
                 w.loc_prev[__ldg(w.loc_h_off + mj) + (x - sh)] = e - sh;
             }
         }
-        if (x == tk.y) {
-            const int32_t sl = atomicAdd(&w.ctrl->n_tips, 1);
-            if (sl < w.tip_cap) w.tips[sl] = tk.y;
-            else atomicOr(&w.ctrl->error, DEV_ERR_CAPACITY);
-        }
+        if (x == tk.y) add_tip(w, tk.y, steps);
     }
     __syncthreads();
     // walk-start marks: frontier, next and prev larger (prev unknown: set
@@ -610,149 +620,162 @@ __global__ void __launch_bounds__(NT, 2048 / NT / IPT) k_label_relink(MeshView m
 }
 
 // ===========================================================================
-// Stages 2-4 fused, one triangle per thread (the same labels, seeds, links,
-// tips and marks as k_label_relink).  A triangle's frontier half-edges form
-// at most one cyclic run among its three (one run, or none, or all three),
-// and only the last half-edge of a run has a successor across a
-// non-frontier edge: a triangle has at most one rotation.  With one
-// triangle per thread, each thread runs its own rotation: a warp's lanes
-// run their rotations side by side without any task list, and every next
-// entry of the CTA is set by its own thread.  prev goes through shared
-// memory (a rotation sets prev[x] for an x of another thread), which also
-// gives the walk-start marks their prev; each warp then stores the next and
-// prev of its 32 triangles as contiguous, coalesced runs.
+// Stages 2-4 fused, one triangle per thread (the same labels, seeds, links
+// and tips as k_label_relink).  A triangle's frontier half-edges form at most
+// one cyclic run among its three (one run, or none, or all three), and only
+// the last half-edge of a run has a successor across a non-frontier edge: a
+// triangle has at most one rotation.  With one triangle per thread, each
+// thread runs its own rotation: a warp's lanes run their rotations side by
+// side without any task list, and every next entry is set by its own thread.
+// prev goes through shared memory (a rotation sets prev[x] for an x of another
+// thread); each warp stores the next and prev of its 32 triangles as
+// contiguous, coalesced runs and shares nothing with the others, so there is no
+// block barrier.  Only the lowest frontier half-edge of a triangle can carry
+// the walk-start mark.
+// Bound by instruction issue together with the latency of its chains of loads
+// (twin, label, twin, label): on the 2048 grid 93 M warp instructions at 3.1 a
+// cycle, 64 warps per SM; with 48 (40 registers) 0.428 ms on the 4096 grid, with
+// 40 0.520 ms, against 0.376 ms here and 0.387 ms with block barriers and a mark
+// test for every half-edge.  Loads without branches (clamped indices past the
+// border) measured 0.407 ms.
 // ===========================================================================
 template <int NT, bool BATCH>
 __global__ void __launch_bounds__(NT, 2048 / NT) k_label_relink1(MeshView m, Work w) {
     static_assert(NT % 32 == 0, "whole warps");
     __shared__ int32_t s_pv[3 * NT];
-    __shared__ int32_t s_nx[3 * NT];
-    __shared__ int32_t s_m0;  // batches: the mesh of the CTA's first triangle
-    const int32_t t0 = blockIdx.x * NT;
+    __shared__ __align__(16) int32_t s_nx[3 * NT];
+    // a warp's 32 triangles and their links are its own: no block barrier
+    const int lane = threadIdx.x & 31;
+    const int32_t t0 = blockIdx.x * NT + ((int32_t)threadIdx.x & ~31);
     const int32_t eb = 3 * t0;
-    const int32_t nE = 3 * min(NT, m.T - t0);
-    const int32_t HI = 3 * m.T;
+    const int32_t nE = 3 * min(32, m.T - t0);  // negative past the mesh's end
+    const uint32_t HI = 3u * (uint32_t)m.T;
     const int32_t lb = 3 * (int32_t)threadIdx.x;
-    const int32_t t = t0 + (int32_t)threadIdx.x;
+    const int32_t t = t0 + lane;
     const bool live = t < m.T;
     const int32_t e0 = 3 * t;
-    if (BATCH && threadIdx.x == 0) s_m0 = mesh_of(w.loc_seg, w.loc_t_off, w.loc_n, t0);
+    int32_t m0 = 0;  // batches: the mesh of the warp's first triangle
+    if (BATCH) {
+        if (lane == 0 && live) m0 = mesh_of(w.loc_seg, w.loc_t_off, w.loc_n, t0);
+        m0 = __shfl_sync(0xffffffffu, m0, 0);
+    }
+    const int32_t ws = 3 * ((int32_t)threadIdx.x & ~31);  // the warp's first slot
     uint32_t F = 0, fl = 0;
     uint32_t kt = 3;          // the local index of the rotating half-edge (3: none)
-    int32_t twk = 0;          // its twin (the rotation coming back to it finds a tip)
-    int32_t ty = 0;           // the rotation: current half-edge 3 ty + lx, ley = le(ty)
-    uint32_t lx = 0, ley = 0;
+    uint32_t kf = 3;          // that of the run's first half-edge (3: no frontier, or all of it)
+    int32_t twk = 0;          // the rotating half-edge's twin (coming back to it finds a tip)
+    uint32_t x = 0, lx = 0, ley = 0;  // the rotation: half-edge, its local index, its triangle's longest
     if (live) {
-        int32_t tw[3], ttri[3];
-        uint32_t tloc[3], lnb[3];
-        tw[0] = __ldg(m.twin + e0);
-        tw[1] = __ldg(m.twin + e0 + 1);
-        tw[2] = __ldg(m.twin + e0 + 2);
+        uint32_t tw[3], ttri[3], tloc[3], lnb[3];
+        tw[0] = (uint32_t)__ldg(m.twin + e0);
+        tw[1] = (uint32_t)__ldg(m.twin + e0 + 1);
+        tw[2] = (uint32_t)__ldg(m.twin + e0 + 2);
         const uint32_t ltl = w.le[t];
         uint32_t twle = 0;
 #pragma unroll
-        for (int k = 0; k < 3; k++) {
+        for (uint32_t k = 0; k < 3; k++) {
             const bool b = tw[k] >= HI;
-            ttri[k] = b ? 0 : div3(tw[k]);
-            tloc[k] = (uint32_t)(tw[k] - 3 * ttri[k]);
-            lnb[k] = b ? 3u : (uint32_t)w.le[ttri[k]];
-            const bool tl = !b && lnb[k] == tloc[k];
-            F |= (uint32_t)(b || ((uint32_t)k != ltl && !tl)) << k;
+            ttri[k] = b ? 0u : tw[k] / 3u;
+            tloc[k] = tw[k] - 3u * ttri[k];
+            lnb[k] = b ? ~0u : (uint32_t)w.le[ttri[k]];
+            const bool tl = lnb[k] == tloc[k];
+            F |= (uint32_t)(b || (k != ltl && !tl)) << k;
             twle |= (uint32_t)tl << k;
         }
-        const int32_t twl = ltl == 0u ? tw[0] : (ltl == 1u ? tw[1] : tw[2]);
-        const bool seed = (twl >= HI) || (((twle >> ltl) & 1u) && (e0 + (int32_t)ltl) < twl);
+        const uint32_t twl = ltl == 0u ? tw[0] : (ltl == 1u ? tw[1] : tw[2]);
+        const bool seed = (twl >= HI) || (((twle >> ltl) & 1u) && (uint32_t)e0 + ltl < twl);
         fl = F | ((uint32_t)seed << 6);
-        // prev of slot j: its triangle link when j is not frontier or its
-        // predecessor in the triangle is frontier; else set by a rotation
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            const int k = j == 0 ? 2 : j - 1;
-            s_pv[lb + j] = (!((F >> j) & 1u) || ((F >> k) & 1u)) ? e0 + k : -1;
-        }
-        // the frontier half-edge whose successor in the triangle is not
-        // frontier: bit k of rot is F bit k + 1 (mod 3), so pend has one bit
-        // at most (1, 2 or 4 -> k = pend >> 1)
-        const uint32_t rot = ((F >> 1) | (F << 2)) & 7u;
-        const uint32_t pend = F & ~rot;
-        if (pend) {
-            kt = pend >> 1;
-            const uint32_t j = kt == 2u ? 0u : kt + 1u;
-            twk = kt == 0u ? tw[0] : (kt == 1u ? tw[1] : tw[2]);
-            ty = j == 0u ? ttri[0] : (j == 1u ? ttri[1] : ttri[2]);
-            const uint32_t ly = j == 0u ? tloc[0] : (j == 1u ? tloc[1] : tloc[2]);
-            ley = j == 0u ? lnb[0] : (j == 1u ? lnb[1] : lnb[2]);
+        // the run's last half-edge (its successor in the triangle is not
+        // frontier) rotates; the first one's predecessor is a rotation's.  One
+        // bit at most: 1, 2 or 4 -> k = bit >> 1 (0 stays 0: told by F)
+        const uint32_t last = F & ~((F >> 1) | (F << 2)), head = F & ~((F << 1) | (F >> 2));
+        s_pv[lb] = head & 1u ? -1 : e0 + 2;
+        s_pv[lb + 1] = head & 2u ? -1 : e0;
+        s_pv[lb + 2] = head & 4u ? -1 : e0 + 1;
+        if (last) {
+            kt = last >> 1;
+            kf = head >> 1;
+            twk = (int32_t)(kt == 0u ? tw[0] : (kt == 1u ? tw[1] : tw[2]));
+            // x = CW(next e) = next(twin(next e)), j = next e's local index
+            const uint32_t txj = kt == 2u ? tw[0] : (kt == 0u ? tw[1] : tw[2]);
+            const uint32_t ly = kt == 2u ? tloc[0] : (kt == 0u ? tloc[1] : tloc[2]);
+            ley = kt == 2u ? lnb[0] : (kt == 0u ? lnb[1] : lnb[2]);
+            x = ly == 2u ? txj - 2u : txj + 1u;
             lx = ly == 2u ? 0u : ly + 1u;
         }
     }
-    __syncthreads();  // every prev slot initialised before rotations write them
+    __syncwarp();  // every prev slot initialised before rotations write them
     int32_t mj = 0, sh = 0;  // batches: the thread's mesh and its first union half-edge
     if (BATCH && live) {
-        mj = s_m0;
+        mj = m0;
         while (mj + 1 < w.loc_n && __ldg(w.loc_t_off + mj + 1) <= t) mj++;
         sh = 3 * __ldg(w.loc_t_off + mj);
     }
-    int32_t x = 3 * ty + (int32_t)lx;
     if (kt < 3u) {
-        // x = CW(next e) = next(twin(next e)); while x is not frontier,
-        // x = CW(x).  The next step's twin is fetched with this step's label.
+        // while x is not frontier, x = CW(x).  The next step's twin is fetched
+        // with this step's label.
         const int32_t e = e0 + (int32_t)kt;
-        int32_t tx = __ldg(m.twin + x);
+        uint32_t tx = (uint32_t)__ldg(m.twin + x);
         int32_t steps = 0;
-        while (true) {
-            if (tx >= HI) break;                     // border edge: frontier
-            const int32_t ttx = div3(tx);
-            const uint32_t ltx = (uint32_t)(tx - 3 * ttx);
-            const uint32_t lxn = ltx == 2u ? 0u : ltx + 1u;
-            const int32_t xn = 3 * ttx + (int32_t)lxn;
+        while (tx < HI) {                            // a border edge is frontier
+            const uint32_t ttx = tx / 3u;
+            const uint32_t ltx = tx - 3u * ttx;
+            const uint32_t xn = ltx == 2u ? tx - 2u : tx + 1u;
             const uint32_t lex = w.le[ttx];
-            const int32_t txn = __ldg(m.twin + xn);
+            const uint32_t txn = (uint32_t)__ldg(m.twin + xn);
             if (ley != lx && lex != ltx) break;      // neither half longest: frontier
             ley = lex;
             x = xn;
-            lx = lxn;
+            lx = xn - 3u * ttx;
             tx = txn;
             if (++steps > w.max_rot) {
                 atomicOr(&w.ctrl->error, DEV_ERR_NONTERMINATING);
                 break;
             }
         }
-        const uint32_t dx = (uint32_t)(x - eb);
-        if (dx < (uint32_t)nE) s_pv[dx] = e;
+        const uint32_t dx = x - (uint32_t)eb;
+        if (dx < 96u) s_pv[ws + (int32_t)dx] = e;  // (past the end of the mesh there is no x)
         else if (!BATCH) m.prev[x] = e;
-        else w.loc_prev[__ldg(w.loc_h_off + mj) + (x - sh)] = e - sh;  // e, x lie in mesh mj
-        if (x == twk) {
-            const int32_t sl = atomicAdd(&w.ctrl->n_tips, 1);
-            if (sl < w.tip_cap) w.tips[sl] = twk;
-            else atomicOr(&w.ctrl->error, DEV_ERR_CAPACITY);
-        }
+        else w.loc_prev[__ldg(w.loc_h_off + mj) + ((int32_t)x - sh)] = e - sh;  // e, x lie in mesh mj
+        if ((int32_t)x == twk) add_tip(w, twk, steps);
     }
-    __syncthreads();  // every prev slot is final
-    // walk-start marks: frontier, next and prev larger (prev -1: set by
-    // another CTA, counted as larger)
+    __syncwarp();  // every prev slot is final
+    // the walk-start mark: next and prev larger (prev -1: set by another warp,
+    // counted as larger).  Only the lowest frontier half-edge can be a
+    // polygon's minimum: links inside the triangle ascend, but for the one from
+    // its third half-edge to its first.
     if (live) {
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            const int32_t e = e0 + k;
-            const int32_t nk = (uint32_t)k == kt ? x : e0 + (k == 2 ? 0 : k + 1);
-            const int32_t pk = s_pv[lb + k];
-            if (((F >> k) & 1u) && nk > e && (pk < 0 || pk > e)) fl |= 8u << k;
-            s_nx[lb + k] = nk;
+        if (F) {
+            const uint32_t kl = F & 1u ? 0u : F >> 1 & 1u ? 1u : 2u;
+            const uint32_t el = (uint32_t)e0 + kl;
+            const uint32_t pk = (uint32_t)s_pv[lb + (int32_t)kl];  // -1 is the largest
+            if ((kl != kt || x > el) && (kl != kf || pk > el)) fl |= 8u << kl;
         }
+        const int32_t xi = (int32_t)x;
+        s_nx[lb] = kt == 0u ? xi : e0 + 1;
+        s_nx[lb + 1] = kt == 1u ? xi : e0 + 2;
+        s_nx[lb + 2] = kt == 2u ? xi : e0;
         w.flags[t] = (uint8_t)fl;
     }
     __syncwarp();
     // each warp stores the links of its 96 half-edges in place, coalesced
     // (in a batch, also in the meshes' own indices and arrays; a batch's
     // union prev is never read, so it is not written)
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int32_t bj = BATCH ? s_m0 : 0;
-    for (int i = lane; i < 96; i += 32) {
-        const int32_t sl = 96 * wid + i;
-        if (sl >= nE) break;
-        const int32_t xe = eb + sl;
-        const int32_t nv = s_nx[sl];
-        const int32_t pv = s_pv[sl];
+    if (!BATCH && nE == 96) {
+        if (lane < 24)
+            reinterpret_cast<int4 *>(m.next + eb)[lane] = reinterpret_cast<const int4 *>(s_nx + ws)[lane];
+        int32_t *pd = m.prev + eb + lane;
+        const int32_t *ps = s_pv + ws + lane;
+#pragma unroll
+        for (int i = 0; i < 96; i += 32)
+            if (ps[i] >= 0) pd[i] = ps[i];
+        return;
+    }
+    int32_t bj = m0;
+    for (int i = lane; i < nE; i += 32) {
+        const int32_t xe = eb + i;
+        const int32_t nv = s_nx[ws + i];
+        const int32_t pv = s_pv[ws + i];
         m.next[xe] = nv;
         if (!BATCH) {
             if (pv >= 0) m.prev[xe] = pv;
