@@ -82,110 +82,129 @@ __device__ int cross_sign(const double2 *__restrict__ xy, const Pt &a, const Pt 
     return c > 0.0 ? 1 : (c < 0.0 ? -1 : 0);
 }
 
-// A slot at the end of a list shared by the whole grid: the lanes of a warp
-// that reach this call together take consecutive slots with one atomic, so
-// the list's counter sees one atomic per warp and call instead of one per
-// entry (a million same-address atomics serialise in L2).  List order is
+// A slot at the end of a list shared by the whole grid for every lane of the
+// (whole) warp that asks for one: one atomic per warp and call.  List order is
 // free: every consumer of these lists treats them as sets.
-__device__ __forceinline__ int32_t append_slot(int32_t *count) {
-    const uint32_t mask = __activemask();
+__device__ __forceinline__ int32_t warp_slot(int32_t *count, bool want) {
+    const uint32_t bal = __ballot_sync(0xffffffffu, want);
     const int lane = (int)(threadIdx.x & 31u);
-    const int leader = __ffs(mask) - 1;
     int32_t base = 0;
-    if (lane == leader) base = atomicAdd(count, __popc(mask));
-    base = __shfl_sync(mask, base, leader);
-    return base + __popc(mask & ((1u << lane) - 1u));
+    if (lane == 0 && bal) base = atomicAdd(count, __popc(bal));
+    return __shfl_sync(0xffffffffu, base, 0) + __popc(bal & ((1u << lane) - 1u));
 }
 
 // ===========================================================================
 // The corners: for a frontier half-edge e = 3t + k, v = target(e) is the
 // triangle's vertex k + 1, origin(e) its vertex k, and the corner's other
-// side is x = next[e].  k_convex_reflex tests every corner (one thread per
-// triangle, its three vertices loaded once, the corners' chains issued
-// together); corner_chords chooses a reflex corner's chords (appended to the
-// list; the frontier bits are set by the next kernel, so every thread reads
-// the frontier of the Polylla mesh).
+// side is x = next[e].  k_convex_reflex tests every corner; k_convex_chords
+// chooses a reflex corner's chords (appended to the list; the frontier bits are
+// set by the next kernel, so every thread reads the frontier of the Polylla
+// mesh).
 // ===========================================================================
-__device__ void corner_chords(const MeshView &m, const Work &w, int32_t e, int32_t x, const Pt &pv, Pt cur,
-                              const Pt &pw, int32_t *list, int32_t *count, int32_t cap) {
-    int32_t y = nx_of(e);
-    int32_t steps = 0;
-    while (cross_sign(m.xy, cur, pw, pv) > 0) {
-        int32_t best = -1;
-        Pt bp = cur;
-        while (y != x) {
-            const Pt pd = load_pt(m.xy, __ldg(m.origin + nx_of(y)));  // target(y)
-            if (cross_sign(m.xy, cur, pd, pv) > 0) break;             // beyond a half turn
-            best = y;
-            bp = pd;
-            y = nx_of(__ldg(m.twin + y));                             // CW(y)
-            if (++steps > w.max_rot) {
-                atomicOr(&w.ctrl->error, DEV_ERR_NONTERMINATING);
-                break;
-            }
+// k_convex_reflex: one thread per triangle; the reflex corners go to a list, so
+// that the chord search (a chain of dependent loads) runs one reflex corner per
+// thread in k_convex_chords instead of holding up a warp of mostly convex
+// corners.  A corner whose successor is the next half-edge of its own triangle
+// is a triangle's angle, less than a half turn: only the last half-edge of the
+// triangle's cyclic run of frontier half-edges has a link across an edge, so a
+// triangle holds at most one reflex corner.  The list's counter takes one atomic
+// per block of CR_THREADS triangles: with one per warp and local half-edge (94 k
+// on 1 M triangles, one after the other in L2) the kernel took 64 us there.
+constexpr int CR_THREADS = 512;
+__global__ void __launch_bounds__(CR_THREADS) k_convex_reflex(MeshView m, Work w, int32_t *reflex, int32_t *n_reflex,
+                                                              int32_t cap) {
+    constexpr int NW = CR_THREADS / 32;
+    __shared__ uint32_t s_n[NW];
+    __shared__ int32_t s_base;
+    const int lane = (int)(threadIdx.x & 31u), wid = (int)(threadIdx.x >> 5);
+    for (int64_t b = (int64_t)blockIdx.x * CR_THREADS; b < m.T; b += (int64_t)gridDim.x * CR_THREADS) {
+        const int64_t t = b + threadIdx.x;
+        const uint32_t F = t < m.T ? w.flags[t] & 7u : 0u;
+        int32_t e = 0;
+        bool is_reflex = false;
+        const uint32_t last = F & ~((F >> 1) | (F << 2));  // one bit at most: 1, 2 or 4
+        if (last) {
+            const int32_t e0 = 3 * (int32_t)t, k = (int32_t)(last >> 1);
+            e = e0 + k;
+            const int32_t x = m.next[e];
+            const Pt pa = load_pt(m.xy, __ldg(m.origin + e));                      // origin(e)
+            const Pt pv = load_pt(m.xy, __ldg(m.origin + e0 + (k == 2 ? 0 : k + 1)));  // target(e)
+            const Pt pw = load_pt(m.xy, __ldg(m.origin + nx_of(x)));               // target(x)
+            is_reflex = cross_sign(m.xy, pa, pw, pv) > 0;
         }
-        if (best < 0 || steps > w.max_rot) return;                    // candidates ran out: left reflex
-        const int32_t slot = append_slot(count);
-        if (slot < cap) list[slot] = best;
-        else atomicOr(&w.ctrl->error, DEV_ERR_CAPACITY);
-        cur = bp;
+        const uint32_t bal = __ballot_sync(0xffffffffu, is_reflex);
+        if (lane == 0) s_n[wid] = (uint32_t)__popc(bal);
+        __syncthreads();
+        if (wid == 0) {
+            const uint32_t n = lane < NW ? s_n[lane] : 0u;
+            uint32_t inc = n;
+#pragma unroll
+            for (int o = 1; o < NW; o <<= 1) {
+                const uint32_t u = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += u;
+            }
+            if (lane < NW) s_n[lane] = inc - n;
+            if (lane == NW - 1) s_base = inc ? atomicAdd(n_reflex, (int32_t)inc) : 0;
+        }
+        __syncthreads();
+        if (is_reflex) {
+            const int32_t slot = s_base + (int32_t)s_n[wid] + __popc(bal & ((1u << lane) - 1u));
+            if (slot < cap) reflex[slot] = e;
+            else atomicOr(&w.ctrl->error, DEV_ERR_CAPACITY);
+        }
+        __syncthreads();  // s_n and s_base are the next round's
     }
 }
 
-// k_convex_reflex: one thread per triangle; the reflex corners of its
-// frontier half-edges go to a list, so that the chord search (a chain of
-// dependent loads) runs one reflex corner per thread in k_convex_chords
-// instead of holding up a warp of mostly convex corners.
-__global__ void __launch_bounds__(256, 4) k_convex_reflex(MeshView m, Work w, int32_t *reflex, int32_t *n_reflex,
-                                                          int32_t cap) {
-    for (int32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < m.T; t += gridDim.x * blockDim.x) {
-        const uint32_t f = w.flags[t] & 7u;
-        if (!f) continue;
-        const int32_t e0 = 3 * t;
-        // a corner whose successor is the next half-edge of its own triangle
-        // is a triangle's angle, less than a half turn: only corners whose
-        // link crossed an edge can be reflex
-        int32_t x[3];
-        uint32_t test = 0;
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            if (!((f >> k) & 1u)) continue;
-            x[k] = m.next[e0 + k];
-            if (x[k] != e0 + (k == 2 ? 0 : k + 1)) test |= 1u << k;
-        }
-        if (!test) continue;
-        Pt p[3];
-#pragma unroll
-        for (int k = 0; k < 3; k++) p[k] = load_pt(m.xy, __ldg(m.origin + e0 + k));
-        Pt pw[3];
-#pragma unroll
-        for (int k = 0; k < 3; k++)
-            if ((test >> k) & 1u) pw[k] = load_pt(m.xy, __ldg(m.origin + nx_of(x[k])));  // target(x)
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            if (!((test >> k) & 1u)) continue;
-            if (cross_sign(m.xy, p[k], pw[k], p[k == 2 ? 0 : k + 1]) > 0) {  // v = target(e): vertex k + 1
-                const int32_t slot = append_slot(n_reflex);
-                if (slot < cap) reflex[slot] = e0 + k;
-                else atomicOr(&w.ctrl->error, DEV_ERR_CAPACITY);
-            }
-        }
-    }
-}
-
-// k_convex_chords: one thread per reflex corner e: its chords
+// k_convex_chords: one thread per reflex corner e: its chords.  A warp's lanes
+// search a chord each and then take their slots together: one atomic per warp
+// and chord.
 __global__ void __launch_bounds__(256) k_convex_chords(MeshView m, Work w, const int32_t *reflex,
                                                        const int32_t *n_reflex, int32_t cap_reflex, int32_t *list,
                                                        int32_t *count, int32_t cap) {
     int32_t n = *n_reflex;
     if (n > cap_reflex) n = cap_reflex;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int32_t e = reflex[i];
-        const int32_t x = m.next[e];
-        const Pt pv = load_pt(m.xy, __ldg(m.origin + nx_of(e)));   // target(e)
-        const Pt pa = load_pt(m.xy, __ldg(m.origin + e));          // origin(e)
-        const Pt pw = load_pt(m.xy, __ldg(m.origin + nx_of(x)));   // target(x)
-        corner_chords(m, w, e, x, pv, pa, pw, list, count, cap);
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = b + threadIdx.x;
+        bool open = i < n;  // the corner left of cur is still reflex
+        int32_t x = 0, y = 0, steps = 0;
+        Pt pv{}, cur{}, pw{};
+        if (open) {
+            const int32_t e = reflex[i];
+            x = m.next[e];
+            y = nx_of(e);
+            pv = load_pt(m.xy, __ldg(m.origin + y));           // target(e)
+            cur = load_pt(m.xy, __ldg(m.origin + e));          // origin(e)
+            pw = load_pt(m.xy, __ldg(m.origin + nx_of(x)));    // target(x)
+        }
+        // (the first test is the one that put the corner on the list)
+        while (__any_sync(0xffffffffu, open)) {
+            int32_t best = -1;
+            if (open) {
+                Pt bp = cur;
+                while (y != x) {
+                    const int32_t ty = __ldg(m.twin + y);
+                    const Pt pd = load_pt(m.xy, __ldg(m.origin + nx_of(y)));  // target(y)
+                    if (cross_sign(m.xy, cur, pd, pv) > 0) break;             // beyond a half turn
+                    best = y;
+                    bp = pd;
+                    y = nx_of(ty);                                            // CW(y)
+                    if (++steps > w.max_rot) {
+                        atomicOr(&w.ctrl->error, DEV_ERR_NONTERMINATING);
+                        break;
+                    }
+                }
+                if (steps > w.max_rot) best = -1;
+                cur = bp;
+            }
+            const int32_t slot = warp_slot(count, best >= 0);
+            if (best >= 0) {
+                if (slot < cap) list[slot] = best;
+                else atomicOr(&w.ctrl->error, DEV_ERR_CAPACITY);
+            }
+            // without a candidate the corner is left reflex
+            open = best >= 0 && cross_sign(m.xy, cur, pw, pv) > 0;
+        }
     }
 }
 
@@ -205,9 +224,9 @@ __global__ void __launch_bounds__(256) k_convex_mark(MeshView m, Work w, const i
 
 void launch_convex_chords(const MeshView &m, const Work &w, int32_t *reflex, int32_t *n_reflex, int32_t *list,
                           int32_t *count, int32_t cap, cudaStream_t s) {
-    const int64_t want = ((int64_t)m.T + 255) / 256;
-    const int blocks = (int)(want < 16 * (int64_t)w.persistent_blocks ? want : 16 * (int64_t)w.persistent_blocks);
-    k_convex_reflex<<<blocks > 0 ? blocks : 1, 256, 0, s>>>(m, w, reflex, n_reflex, cap);
+    const int64_t want = ((int64_t)m.T + CR_THREADS - 1) / CR_THREADS;
+    const int64_t most = 16 * (int64_t)w.persistent_blocks;
+    k_convex_reflex<<<(int)(want < most ? want : most), CR_THREADS, 0, s>>>(m, w, reflex, n_reflex, cap);
     k_convex_chords<<<8 * w.persistent_blocks, 256, 0, s>>>(m, w, reflex, n_reflex, cap, list, count, cap);
 }
 

@@ -52,8 +52,17 @@ __global__ void __launch_bounds__(256) k_chords(MeshView m, Work w) {
     }
 }
 
+// Blocks of a kernel over a list of unknown length: one per `per` triangles (a
+// list longer than that takes the kernel's loop more often), at most the chip
+// full.  608 blocks for whatever mesh cost the smallest ones their launch, and
+// the links of 500 k chords three rounds.
+static int list_blocks(const MeshView &m, const Work &w, int32_t per) {
+    const int64_t want = m.T / per + 1, most = 2 * (int64_t)w.persistent_blocks;
+    return (int)(want < most ? want : most);
+}
+
 void launch_chords(const MeshView &m, const Work &w, cudaStream_t s) {
-    k_chords<<<w.persistent_blocks, 256, 0, s>>>(m, w);
+    k_chords<<<list_blocks(m, w, 8192), 256, 0, s>>>(m, w);  // random meshes: a tip per 120 triangles
 }
 
 // ===========================================================================
@@ -145,12 +154,12 @@ __global__ void __launch_bounds__(256) k_chord_links(MeshView m, Work w, const i
 }
 
 void launch_chord_links(const MeshView &m, const Work &w, cudaStream_t s) {
-    k_chord_links<<<w.persistent_blocks, 256, 0, s>>>(m, w, w.chords, &w.ctrl->n_tips, w.tip_cap);
+    k_chord_links<<<list_blocks(m, w, 2048), 256, 0, s>>>(m, w, w.chords, &w.ctrl->n_tips, w.tip_cap);
 }
 
 void launch_chord_links_list(const MeshView &m, const Work &w, const int32_t *list, const int32_t *count,
                              int32_t cap, cudaStream_t s) {
-    k_chord_links<<<w.persistent_blocks, 256, 0, s>>>(m, w, list, count, cap);
+    k_chord_links<<<list_blocks(m, w, 512), 256, 0, s>>>(m, w, list, count, cap);  // a chord per 10 to 25 triangles
 }
 
 }  // namespace polylla
