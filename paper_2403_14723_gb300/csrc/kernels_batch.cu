@@ -190,6 +190,8 @@ __global__ void __launch_bounds__(BP_THREADS) k_batch_pack(BatchView b, int32_t 
 // ===========================================================================
 __global__ void k_batch_meta(BatchView b, const int32_t *offsets, const int32_t *poly_off, int32_t *local_offsets,
                              int32_t *meta) {
+    chain_next();
+    chain_wait();
     const int32_t n = b.n;
     const int32_t gt = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
     for (int32_t i = gt; i < n; i += gs) {
@@ -231,8 +233,8 @@ void launch_batch_seg(const int32_t *t_off, int32_t n, int32_t T, int32_t *seg, 
 }
 
 void launch_batch_meta(const BatchView &b, const Work &w, const int32_t *poly_off, int32_t *local_offsets,
-                       int32_t *meta, cudaStream_t s) {
-    k_batch_meta<<<w.persistent_blocks, 256, 0, s>>>(b, w.offsets, poly_off, local_offsets, meta);
+                       int32_t *meta, cudaStream_t s, bool chained) {
+    launch_kernel(k_batch_meta, w.persistent_blocks, 256, 0, s, chained, b, w.offsets, poly_off, local_offsets, meta);
 }
 
 void launch_batch_pack(const BatchView &b, int32_t *u_origin, int32_t *u_twin, int32_t *u_next, int32_t *u_prev,

@@ -116,6 +116,8 @@ __global__ void __launch_bounds__(CR_THREADS) k_convex_reflex(MeshView m, Work w
     constexpr int NW = CR_THREADS / 32;
     __shared__ uint32_t s_n[NW];
     __shared__ int32_t s_base;
+    chain_next();
+    chain_wait();
     const int lane = (int)(threadIdx.x & 31u), wid = (int)(threadIdx.x >> 5);
     for (int64_t b = (int64_t)blockIdx.x * CR_THREADS; b < m.T; b += (int64_t)gridDim.x * CR_THREADS) {
         const int64_t t = b + threadIdx.x;
@@ -162,6 +164,8 @@ __global__ void __launch_bounds__(CR_THREADS) k_convex_reflex(MeshView m, Work w
 __global__ void __launch_bounds__(256) k_convex_chords(MeshView m, Work w, const int32_t *reflex,
                                                        const int32_t *n_reflex, int32_t cap_reflex, int32_t *list,
                                                        int32_t *count, int32_t cap) {
+    chain_next();
+    chain_wait();
     int32_t n = *n_reflex;
     if (n > cap_reflex) n = cap_reflex;
     for (int64_t b = (int64_t)blockIdx.x * blockDim.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
@@ -211,6 +215,8 @@ __global__ void __launch_bounds__(256) k_convex_chords(MeshView m, Work w, const
 // both halves of every listed chord join the frontier (F bits of flags)
 __global__ void __launch_bounds__(256) k_convex_mark(MeshView m, Work w, const int32_t *list, const int32_t *count,
                                                      int32_t cap) {
+    chain_next();
+    chain_wait();
     int32_t n = *count;
     if (n > cap) n = cap;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * n; i += gridDim.x * blockDim.x) {
@@ -223,16 +229,17 @@ __global__ void __launch_bounds__(256) k_convex_mark(MeshView m, Work w, const i
 }
 
 void launch_convex_chords(const MeshView &m, const Work &w, int32_t *reflex, int32_t *n_reflex, int32_t *list,
-                          int32_t *count, int32_t cap, cudaStream_t s) {
+                          int32_t *count, int32_t cap, cudaStream_t s, bool chained) {
     const int64_t want = ((int64_t)m.T + CR_THREADS - 1) / CR_THREADS;
     const int64_t most = 16 * (int64_t)w.persistent_blocks;
-    k_convex_reflex<<<(int)(want < most ? want : most), CR_THREADS, 0, s>>>(m, w, reflex, n_reflex, cap);
-    k_convex_chords<<<8 * w.persistent_blocks, 256, 0, s>>>(m, w, reflex, n_reflex, cap, list, count, cap);
+    launch_kernel(k_convex_reflex, want < most ? want : most, CR_THREADS, 0, s, chained, m, w, reflex, n_reflex, cap);
+    launch_kernel(k_convex_chords, 8 * w.persistent_blocks, 256, 0, s, true, m, w, reflex, n_reflex, cap, list, count,
+                  cap);
 }
 
 void launch_convex_mark(const MeshView &m, const Work &w, const int32_t *list, const int32_t *count, int32_t cap,
-                        cudaStream_t s) {
-    k_convex_mark<<<w.persistent_blocks, 256, 0, s>>>(m, w, list, count, cap);
+                        cudaStream_t s, bool chained) {
+    launch_kernel(k_convex_mark, w.persistent_blocks, 256, 0, s, chained, m, w, list, count, cap);
 }
 
 }  // namespace polylla

@@ -164,6 +164,8 @@ __global__ void __launch_bounds__(LE_THREADS) k_longest_edge(MeshView m, Work w)
     constexpr int LE_TILE = 32 * PER;
     __shared__ __align__(128) int32_t s_org[NW][2][3 * LE_TILE];
     __shared__ __align__(8) uint64_t s_bar[NW][2];
+    chain_next();
+    chain_wait();
     // reset this generate's control block (error word, tip count, totals)
     // and the output tiles' totals
     const int32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -262,6 +264,8 @@ __global__ void __launch_bounds__(LE_THREADS) k_longest_edge_batch(MeshView m, W
     __shared__ __align__(128) int32_t s_tw[NW][2][SPAN];
     __shared__ __align__(8) uint64_t s_bar[NW][2];
     __shared__ int32_t s_r[NW][2], s_j[NW][2];  // per stage: start offset (-1: plain loads), mesh
+    chain_next();
+    chain_wait();
     const int32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
     if (gtid < (int32_t)(sizeof(DevCtrl) / sizeof(int32_t))) reinterpret_cast<int32_t *>(w.ctrl)[gtid] = 0;
     for (int32_t i = gtid; i < w.n_tile_max; i += gridDim.x * blockDim.x) w.tile_state[i] = 0ull;
@@ -374,16 +378,16 @@ int longest_edge_batch_blocks_per_sm() {
     return n > 0 ? n : 1;
 }
 
-void launch_longest_edge(const MeshView &m, const Work &w, cudaStream_t s) {
+void launch_longest_edge(const MeshView &m, const Work &w, cudaStream_t s, bool chained) {
     const int32_t tile = 32 * (w.le_items == 4 && w.loc_n == 0 ? 4 : 2);  // batches: 2 per lane
     const int32_t n_tiles = (m.T + tile - 1) / tile;
     const int32_t want = (n_tiles + LE_THREADS / 32 - 1) / (LE_THREADS / 32);  // one tile per warp
     const int32_t grid = w.loc_n > 0 ? w.le_batch_blocks : w.le_blocks;  // persistent: every CTA resident
     const int blocks = want < grid ? want : grid;
     // the control-block reset needs >= 8 threads: any grid >= 1 works
-    if (w.loc_n > 0) k_longest_edge_batch<2><<<blocks, LE_THREADS, 0, s>>>(m, w);
-    else if (w.le_items == 4) k_longest_edge<4><<<blocks, LE_THREADS, 0, s>>>(m, w);
-    else k_longest_edge<2><<<blocks, LE_THREADS, 0, s>>>(m, w);
+    if (w.loc_n > 0) launch_kernel(k_longest_edge_batch<2>, blocks, LE_THREADS, 0, s, chained, m, w);
+    else if (w.le_items == 4) launch_kernel(k_longest_edge<4>, blocks, LE_THREADS, 0, s, chained, m, w);
+    else launch_kernel(k_longest_edge<2>, blocks, LE_THREADS, 0, s, chained, m, w);
 }
 
 
@@ -450,6 +454,8 @@ __global__ void __launch_bounds__(NT, 2048 / NT / IPT) k_label_relink(MeshView m
     __shared__ __align__(16) int32_t s_pv[3 * TT];
     __shared__ int4 s_task[NT / 32][96 * IPT];
     __shared__ int32_t s_m0;  // batches: the mesh of the CTA's first triangle
+    chain_next();
+    chain_wait();
     const int32_t t0 = blockIdx.x * TT;
     const int32_t nT = min(TT, m.T - t0);
     const int32_t eb = 3 * t0;
@@ -644,6 +650,8 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_label_relink1(MeshView m, Wor
     static_assert(NT % 32 == 0, "whole warps");
     __shared__ int32_t s_pv[3 * NT];
     __shared__ __align__(16) int32_t s_nx[3 * NT];
+    chain_next();
+    chain_wait();
     // a warp's 32 triangles and their links are its own: no block barrier
     const int lane = threadIdx.x & 31;
     const int32_t t0 = blockIdx.x * NT + ((int32_t)threadIdx.x & ~31);
@@ -813,25 +821,25 @@ bool relink_config_valid(int32_t tile, int32_t items) {
 
 int relink_configure() { return 0; }  // static shared memory only
 
-void launch_label_relink(const MeshView &m, const Work &w, cudaStream_t s) {
+void launch_label_relink(const MeshView &m, const Work &w, cudaStream_t s, bool chained) {
 #define X(N)                                                                         \
     if (w.rl_tile == N && w.rl_items == 1) {                                         \
-        if (w.loc_n > 0) k_label_relink1<N, true><<<(m.T + N - 1) / N, N, 0, s>>>(m, w); \
-        else k_label_relink1<N, false><<<(m.T + N - 1) / N, N, 0, s>>>(m, w);       \
+        if (w.loc_n > 0) launch_kernel(k_label_relink1<N, true>, (m.T + N - 1) / N, N, 0, s, chained, m, w); \
+        else launch_kernel(k_label_relink1<N, false>, (m.T + N - 1) / N, N, 0, s, chained, m, w);       \
         return;                                                                      \
     }
     RELINK1_CONFIGS(X)
 #undef X
 #define X(N, I)                                                                      \
     if (w.rl_tile == N * I && w.rl_items == I) {                                     \
-        if (w.loc_n > 0) k_label_relink<N, I, true><<<(m.T + N * I - 1) / (N * I), N, 0, s>>>(m, w);  \
-        else k_label_relink<N, I, false><<<(m.T + N * I - 1) / (N * I), N, 0, s>>>(m, w);        \
+        if (w.loc_n > 0) launch_kernel(k_label_relink<N, I, true>, (m.T + N * I - 1) / (N * I), N, 0, s, chained, m, w);  \
+        else launch_kernel(k_label_relink<N, I, false>, (m.T + N * I - 1) / (N * I), N, 0, s, chained, m, w);        \
         return;                                                                      \
     }
     RELINK_CONFIGS(X)
 #undef X
-    if (w.loc_n > 0) k_label_relink1<128, true><<<(m.T + 127) / 128, 128, 0, s>>>(m, w);
-    else k_label_relink1<128, false><<<(m.T + 127) / 128, 128, 0, s>>>(m, w);
+    if (w.loc_n > 0) launch_kernel(k_label_relink1<128, true>, (m.T + 127) / 128, 128, 0, s, chained, m, w);
+    else launch_kernel(k_label_relink1<128, false>, (m.T + 127) / 128, 128, 0, s, chained, m, w);
 }
 
 }  // namespace polylla

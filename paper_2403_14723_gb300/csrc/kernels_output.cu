@@ -181,6 +181,8 @@ __global__ void __launch_bounds__(TILE / (2 * IPT)) k_poly_count(MeshView m, Wor
     const uint32_t ne = (uint32_t)(3 * nt);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint32_t below = (1u << lane) - 1u;
+    chain_next();
+    chain_wait();
     if (threadIdx.x == 0) {
         mbar_init(&s_bar, 1);
         fence_mbar_init();
@@ -349,6 +351,8 @@ __global__ void __launch_bounds__(TILE / (2 * IPT)) k_poly_count(MeshView m, Wor
 __global__ void __launch_bounds__(SCAN_THREADS) k_tile_scan(MeshView m, Work w, int32_t n) {
     __shared__ unsigned long long s_warp[33];
     __shared__ int s_last;
+    chain_next();
+    chain_wait();
     const int32_t i = blockIdx.x * SCAN_THREADS + threadIdx.x;
     const unsigned long long v = i < n ? w.tile_state[i] : 0ull;
     unsigned long long total;
@@ -437,6 +441,8 @@ __global__ void __launch_bounds__(TILE / IPT, TILE == 1024 && IPT == 4 ? 6 : 1) 
     // batches: the mesh of the tile's first triangle, and where the tile's
     // origins start in s_org (-1: not bulk-copied, loaded below)
     __shared__ int32_t s_j0, s_r;
+    chain_next();
+    chain_wait();
     if (threadIdx.x == 0) {
         mbar_init(&s_bar, 1);
         fence_mbar_init();
@@ -781,36 +787,36 @@ int polygons_blocks_per_sm(int32_t tile, int32_t items) {
 
 // the two kernels of the output stage (an unknown configuration takes the
 // default one: the tuning entry points accept only valid ones)
-void launch_poly_count(const MeshView &m, const Work &w, cudaStream_t s) {
+void launch_poly_count(const MeshView &m, const Work &w, cudaStream_t s, bool chained) {
 #define X(TL, N)                                                                            \
     if (w.out_tile == TL && w.out_items == N) {                                        \
-        k_poly_count<TL, N><<<(m.T + TL - 1) / TL, TL / (2 * N), count_smem<TL, N>(), s>>>(m, w);         \
+        launch_kernel(k_poly_count<TL, N>, (m.T + TL - 1) / TL, TL / (2 * N), count_smem<TL, N>(), s, chained, m, w);         \
         return;                                                                             \
     }
     POLYGON_CONFIGS(X)
 #undef X
     constexpr int TL = OUT_TILE_DEFAULT, N = OUT_ITEMS_DEFAULT;
-    k_poly_count<TL, N><<<(m.T + TL - 1) / TL, TL / (2 * N), count_smem<TL, N>(), s>>>(m, w);
+    launch_kernel(k_poly_count<TL, N>, (m.T + TL - 1) / TL, TL / (2 * N), count_smem<TL, N>(), s, chained, m, w);
 }
 
-void launch_tile_scan(const MeshView &m, const Work &w, cudaStream_t s) {
+void launch_tile_scan(const MeshView &m, const Work &w, cudaStream_t s, bool chained) {
     const int32_t tile = polygons_config_valid(w.out_tile, w.out_items) ? w.out_tile : OUT_TILE_DEFAULT;
     const int32_t n = (m.T + tile - 1) / tile;
-    k_tile_scan<<<(n + SCAN_THREADS - 1) / SCAN_THREADS, SCAN_THREADS, 0, s>>>(m, w, n);
+    launch_kernel(k_tile_scan, (n + SCAN_THREADS - 1) / SCAN_THREADS, SCAN_THREADS, 0, s, chained, m, w, n);
 }
 
-void launch_poly_list(const MeshView &m, const Work &w, cudaStream_t s) {
+void launch_poly_list(const MeshView &m, const Work &w, cudaStream_t s, bool chained) {
 #define X(TL, N)                                                                            \
     if (w.out_tile == TL && w.out_items == N) {                                        \
-        if (w.loc_n > 0) k_poly_list<TL, N, true><<<(m.T + TL - 1) / TL, TL / N, list_smem<TL, N>(), s>>>(m, w); \
-        else k_poly_list<TL, N, false><<<(m.T + TL - 1) / TL, TL / N, list_smem<TL, N>(), s>>>(m, w);      \
+        if (w.loc_n > 0) launch_kernel(k_poly_list<TL, N, true>, (m.T + TL - 1) / TL, TL / N, list_smem<TL, N>(), s, chained, m, w); \
+        else launch_kernel(k_poly_list<TL, N, false>, (m.T + TL - 1) / TL, TL / N, list_smem<TL, N>(), s, chained, m, w);      \
         return;                                                                             \
     }
     POLYGON_CONFIGS(X)
 #undef X
     constexpr int TL = OUT_TILE_DEFAULT, N = OUT_ITEMS_DEFAULT;
-    if (w.loc_n > 0) k_poly_list<TL, N, true><<<(m.T + TL - 1) / TL, TL / N, list_smem<TL, N>(), s>>>(m, w);
-    else k_poly_list<TL, N, false><<<(m.T + TL - 1) / TL, TL / N, list_smem<TL, N>(), s>>>(m, w);
+    if (w.loc_n > 0) launch_kernel(k_poly_list<TL, N, true>, (m.T + TL - 1) / TL, TL / N, list_smem<TL, N>(), s, chained, m, w);
+    else launch_kernel(k_poly_list<TL, N, false>, (m.T + TL - 1) / TL, TL / N, list_smem<TL, N>(), s, chained, m, w);
 }
 
 }  // namespace polylla

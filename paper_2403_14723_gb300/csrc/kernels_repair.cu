@@ -31,6 +31,8 @@ __device__ __forceinline__ void set_start(uint8_t *flags, int32_t e) { set_flag_
 // degree here, to 8 us on 1 M random points (16.8 k tips).
 // ===========================================================================
 __global__ void __launch_bounds__(256) k_chords(MeshView m, Work w) {
+    chain_next();
+    chain_wait();
     int32_t n = w.ctrl->n_tips;
     if (n > w.tip_cap) n = w.tip_cap;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -61,8 +63,8 @@ static int list_blocks(const MeshView &m, const Work &w, int32_t per) {
     return (int)(want < most ? want : most);
 }
 
-void launch_chords(const MeshView &m, const Work &w, cudaStream_t s) {
-    k_chords<<<list_blocks(m, w, 8192), 256, 0, s>>>(m, w);  // random meshes: a tip per 120 triangles
+void launch_chords(const MeshView &m, const Work &w, cudaStream_t s, bool chained) {
+    launch_kernel(k_chords, list_blocks(m, w, 8192), 256, 0, s, chained, m, w);  // random meshes: a tip per 120 triangles
 }
 
 // ===========================================================================
@@ -140,6 +142,8 @@ __device__ __forceinline__ void relink_around(const MeshView &m, const Work &w, 
 // thread follows one chain of loads.
 __global__ void __launch_bounds__(256) k_chord_links(MeshView m, Work w, const int32_t *list, const int32_t *count,
                                                      int32_t cap) {
+    chain_next();
+    chain_wait();
     const int32_t HI = 3 * m.T;
     int32_t n = *count;
     if (n > cap) n = cap;
@@ -153,13 +157,13 @@ __global__ void __launch_bounds__(256) k_chord_links(MeshView m, Work w, const i
     }
 }
 
-void launch_chord_links(const MeshView &m, const Work &w, cudaStream_t s) {
-    k_chord_links<<<list_blocks(m, w, 2048), 256, 0, s>>>(m, w, w.chords, &w.ctrl->n_tips, w.tip_cap);
+void launch_chord_links(const MeshView &m, const Work &w, cudaStream_t s, bool chained) {
+    launch_kernel(k_chord_links, list_blocks(m, w, 2048), 256, 0, s, chained, m, w, w.chords, &w.ctrl->n_tips, w.tip_cap);
 }
 
 void launch_chord_links_list(const MeshView &m, const Work &w, const int32_t *list, const int32_t *count,
-                             int32_t cap, cudaStream_t s) {
-    k_chord_links<<<list_blocks(m, w, 512), 256, 0, s>>>(m, w, list, count, cap);  // a chord per 10 to 25 triangles
+                             int32_t cap, cudaStream_t s, bool chained) {
+    launch_kernel(k_chord_links, list_blocks(m, w, 512), 256, 0, s, chained, m, w, list, count, cap);  // a chord per 10 to 25 triangles
 }
 
 }  // namespace polylla

@@ -431,22 +431,26 @@ static int enqueue(polylla_ctx *c, cudaStream_t s, bool timing) {
         return timing ? cudaEventRecord(c->ev_begin[i], s) : cudaSuccess;
     };
     auto end = [&](int i) -> cudaError_t { return timing ? cudaEventRecord(c->ev_end[i], s) : cudaSuccess; };
-    void (*stages[kCore])(const MeshView &, const Work &, cudaStream_t) = {
+    void (*stages[kCore])(const MeshView &, const Work &, cudaStream_t, bool) = {
         launch_longest_edge, launch_label_relink, launch_chords, launch_chord_links, launch_poly_count,
         launch_tile_scan, launch_poly_list,
     };
+    // a stage is chained to the one before unless an event lies between them
+    bool chained = false;
     for (int i = 0; i < kCore; i++) {
         if (i == 1 && c->wait_before_relink) CK(cudaStreamWaitEvent(s, c->wait_before_relink, 0));
+        if (i == 1 && c->wait_before_relink) chained = false;
         CK(begin(i));
-        stages[i](c->mesh, c->w, s);
+        stages[i](c->mesh, c->w, s, chained);
         CK(end(i));
+        chained = !timing && !(i == 3 && c->record_after_links);
         if (i == 3 && c->record_after_links) CK(cudaEventRecord(c->record_after_links, s));
     }
     if (c->is_batch) {
         CK(begin(kMeta));
         // the relink and repair kernels wrote the meshes' own next/prev and
         // the listing kernel their seeds and polygon ranges
-        if (c->serve) launch_batch_meta(c->bv, c->w, c->poly_off, c->local_offsets, c->meta, s);
+        if (c->serve) launch_batch_meta(c->bv, c->w, c->poly_off, c->local_offsets, c->meta, s, chained);
         CK(end(kMeta));
     }
     c->launches = kKernels + (c->serve ? 1 : 0);
@@ -880,12 +884,13 @@ int polylla_convexify(polylla_ctx *c, polylla_stream stream) {
     CK(cudaMemsetAsync(c->cv_count, 0, 2 * sizeof(int32_t), s));
     CK(cudaMemsetAsync(c->w.tile_state, 0, sizeof(unsigned long long) * (size_t)c->w.n_tile_max, s));
     CK(cudaMemsetAsync(&c->w.ctrl->scan_done, 0, 2 * sizeof(int32_t), s));  // and cross_used
-    launch_convex_chords(c->mesh, c->w, c->cv_reflex, c->cv_count + 1, c->cv_list, c->cv_count, c->cv_cap, s);
-    launch_convex_mark(c->mesh, c->w, c->cv_list, c->cv_count, c->cv_cap, s);
-    launch_chord_links_list(c->mesh, c->w, c->cv_list, c->cv_count, c->cv_cap, s);
-    launch_poly_count(c->mesh, c->w, s);
-    launch_tile_scan(c->mesh, c->w, s);
-    launch_poly_list(c->mesh, c->w, s);
+    launch_convex_chords(c->mesh, c->w, c->cv_reflex, c->cv_count + 1, c->cv_list, c->cv_count, c->cv_cap, s,
+                         false);
+    launch_convex_mark(c->mesh, c->w, c->cv_list, c->cv_count, c->cv_cap, s, true);
+    launch_chord_links_list(c->mesh, c->w, c->cv_list, c->cv_count, c->cv_cap, s, true);
+    launch_poly_count(c->mesh, c->w, s, true);
+    launch_tile_scan(c->mesh, c->w, s, true);
+    launch_poly_list(c->mesh, c->w, s, true);
     CK(cudaGetLastError());
     return POLYLLA_OK;
 }

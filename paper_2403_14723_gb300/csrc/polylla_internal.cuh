@@ -155,6 +155,34 @@ constexpr int RL_ITEMS_DEFAULT = 1;
 // bounded waits: iterations of an mbarrier try_wait loop before giving up
 constexpr int MBAR_WAIT_LIMIT = 1 << 22;
 
+// ---- launches that follow one another (programmatic dependent launch) --------
+// The kernels of a generate each need all of the one before.  Launched plainly,
+// each starts only when its predecessor has drained: 1 to 2 us of an idle chip
+// per kernel, most of a small mesh's time.  A chained launch may be set up while
+// its predecessor still runs: every kernel of the chain first lets its successor
+// in (chain_next), whose blocks take what room is left on the SMs and wait there
+// (chain_wait: until the predecessor has ended and its writes are visible).
+// Every thread waits before it touches global memory, so a kernel has ended only
+// after all kernels before it; without a chained launch both are no-ops.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// chained only directly behind a kernel of the chain on the same stream
+template <typename... P, typename... A>
+void launch_kernel(void (*kernel)(P...), int64_t blocks, int threads, size_t smem, cudaStream_t s, bool chained,
+                   const A &...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // an error stays pending for the caller's check
+}
+
 // ---- bulk copies (TMA engine) and mbarriers, inline PTX --------------------
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -255,30 +283,31 @@ __device__ __forceinline__ int32_t pv_of(int32_t e) {
     return b + (k == 0 ? 2 : k - 1);
 }
 
-// launchers (each enqueues one kernel on stream)
+// launchers (each enqueues one kernel on stream; chained: behind a kernel of
+// the chain, see launch_kernel)
 void launch_validate(const MeshView &m, int32_t *bad, cudaStream_t s);
-void launch_longest_edge(const MeshView &m, const Work &w, cudaStream_t s);
+void launch_longest_edge(const MeshView &m, const Work &w, cudaStream_t s, bool chained);
 int longest_edge_blocks_per_sm(int32_t items);
 int longest_edge_batch_blocks_per_sm();
-void launch_label_relink(const MeshView &m, const Work &w, cudaStream_t s);
+void launch_label_relink(const MeshView &m, const Work &w, cudaStream_t s, bool chained);
 // allows the relink kernels their shared memory on the current device (once
 // per device before the first launch); 0 on success
 int relink_configure();
 bool relink_config_valid(int32_t tile, int32_t items);
-void launch_chords(const MeshView &m, const Work &w, cudaStream_t s);
-void launch_chord_links(const MeshView &m, const Work &w, cudaStream_t s);
+void launch_chords(const MeshView &m, const Work &w, cudaStream_t s, bool chained);
+void launch_chord_links(const MeshView &m, const Work &w, cudaStream_t s, bool chained);
 void launch_chord_links_list(const MeshView &m, const Work &w, const int32_t *list, const int32_t *count,
-                             int32_t cap, cudaStream_t s);
+                             int32_t cap, cudaStream_t s, bool chained);
 // convexification (kernels_convex.cu)
 // two kernels: the reflex corners into reflex (count n_reflex), then their
 // chords into list (count count); both lists hold at most cap entries
 void launch_convex_chords(const MeshView &m, const Work &w, int32_t *reflex, int32_t *n_reflex, int32_t *list,
-                          int32_t *count, int32_t cap, cudaStream_t s);
+                          int32_t *count, int32_t cap, cudaStream_t s, bool chained);
 void launch_convex_mark(const MeshView &m, const Work &w, const int32_t *list, const int32_t *count, int32_t cap,
-                        cudaStream_t s);
-void launch_poly_count(const MeshView &m, const Work &w, cudaStream_t s);
-void launch_tile_scan(const MeshView &m, const Work &w, cudaStream_t s);
-void launch_poly_list(const MeshView &m, const Work &w, cudaStream_t s);
+                        cudaStream_t s, bool chained);
+void launch_poly_count(const MeshView &m, const Work &w, cudaStream_t s, bool chained);
+void launch_tile_scan(const MeshView &m, const Work &w, cudaStream_t s, bool chained);
+void launch_poly_list(const MeshView &m, const Work &w, cudaStream_t s, bool chained);
 // allows the output kernels their shared memory on the current device (once
 // per device before the first launch); 0 on success
 int polygons_configure();
@@ -298,6 +327,6 @@ void launch_batch_pack(const BatchView &b, int32_t *u_origin, int32_t *u_twin, i
                        int32_t *bad, int32_t *input_err, cudaStream_t s);
 void launch_batch_seg(const int32_t *t_off, int32_t n, int32_t T, int32_t *seg, cudaStream_t s);
 void launch_batch_meta(const BatchView &b, const Work &w, const int32_t *poly_off, int32_t *local_offsets,
-                       int32_t *meta, cudaStream_t s);
+                       int32_t *meta, cudaStream_t s, bool chained);
 
 }  // namespace polylla

@@ -140,13 +140,13 @@ extern "C" int polylla_generate_noalloc(const polylla_mesh *mesh, int32_t *seeds
     // before it is read, so the previous call's contents never leak into
     // this one.
     cudaStream_t s = (cudaStream_t)stream;
-    launch_longest_edge(m, w, s);
-    launch_label_relink(m, w, s);
-    launch_chords(m, w, s);
-    launch_chord_links(m, w, s);
-    launch_poly_count(m, w, s);
-    launch_tile_scan(m, w, s);
-    launch_poly_list(m, w, s);
+    launch_longest_edge(m, w, s, false);
+    launch_label_relink(m, w, s, true);
+    launch_chords(m, w, s, true);
+    launch_chord_links(m, w, s, true);
+    launch_poly_count(m, w, s, true);
+    launch_tile_scan(m, w, s, true);
+    launch_poly_list(m, w, s, true);
     // status3 = {P, N_F, device error bits}, copied device to device
     if (cudaMemcpyAsync(status3, &w.ctrl->n_polygons, 2 * sizeof(int32_t), cudaMemcpyDeviceToDevice, s) !=
             cudaSuccess ||
