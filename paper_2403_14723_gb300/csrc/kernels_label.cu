@@ -254,6 +254,24 @@ __global__ void __launch_bounds__(LE_THREADS) k_longest_edge(MeshView m, Work w)
 // the longest edge as on a single mesh, from the coordinates at the mesh's
 // vertex offset.
 // ===========================================================================
+// what a triangle of a mesh needs of the batch's tables: the mesh's first and
+// number of interior union half-edges, local entries, vertices, and the shift
+// of its border half-edges into the union
+struct MeshRow {
+    int32_t t3, ti3, h0, hi, v0, vi, bo;
+};
+__device__ __forceinline__ MeshRow mesh_row(const Work &w, int32_t j, int32_t HI) {
+    MeshRow r;
+    r.t3 = 3 * __ldg(w.loc_t_off + j);
+    r.ti3 = 3 * __ldg(w.loc_t_off + j + 1) - r.t3;
+    r.h0 = __ldg(w.loc_h_off + j);
+    r.hi = __ldg(w.loc_h_off + j + 1) - r.h0;
+    r.v0 = __ldg(w.loc_v_off + j);
+    r.vi = __ldg(w.loc_v_off + j + 1) - r.v0;
+    r.bo = HI + (r.h0 - r.t3) - r.ti3;
+    return r;
+}
+
 template <int PER>
 __global__ void __launch_bounds__(LE_THREADS) k_longest_edge_batch(MeshView m, Work w) {
     constexpr int NW = LE_THREADS / 32;
@@ -263,7 +281,8 @@ __global__ void __launch_bounds__(LE_THREADS) k_longest_edge_batch(MeshView m, W
     __shared__ __align__(128) int32_t s_org[NW][2][SPAN];
     __shared__ __align__(128) int32_t s_tw[NW][2][SPAN];
     __shared__ __align__(8) uint64_t s_bar[NW][2];
-    __shared__ int32_t s_r[NW][2], s_j[NW][2];  // per stage: start offset (-1: plain loads), mesh
+    __shared__ int32_t s_r[NW][2];        // per stage: start offset (-1: plain loads)
+    __shared__ MeshRow s_row[NW][2];      // and the mesh of a bulk-copied tile
     chain_next();
     chain_wait();
     const int32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -286,10 +305,11 @@ __global__ void __launch_bounds__(LE_THREADS) k_longest_edge_batch(MeshView m, W
         const int32_t j = mesh_of(w.loc_seg, w.loc_t_off, w.loc_n, t0);
         const int32_t t3 = 3 * __ldg(w.loc_t_off + j);
         const bool one = w.loc_aligned && 3 * __ldg(w.loc_t_off + j + 1) >= 3 * (t0 + nt);
-        s_j[warp][st] = j;
         fence_proxy_async_smem();
         if (one) {
-            const int32_t L0 = __ldg(w.loc_h_off + j) + (3 * t0 - t3);
+            const MeshRow row = mesh_row(w, j, HI);
+            s_row[warp][st] = row;
+            const int32_t L0 = row.h0 + (3 * t0 - t3);
             const int32_t r = L0 & 3;
             const uint32_t bytes = ((uint32_t)(r + 3 * nt) * 4u + 15u) & ~15u;
             s_r[warp][st] = r;
@@ -324,18 +344,15 @@ __global__ void __launch_bounds__(LE_THREADS) k_longest_edge_batch(MeshView m, W
         const int32_t *stw = s_tw[warp][st] + (r > 0 ? r : 0);
         double2 p[PER][3];
         int32_t tw[PER][3];
+        MeshRow row{};
+        if (r >= 0) row = s_row[warp][st];
 #pragma unroll
         for (int q = 0; q < PER; q++) {
             const int32_t lt = lane + 32 * q;
             const int32_t t = t0 + lt;
             if (t >= m.T) continue;
-            const int32_t j = r >= 0 ? s_j[warp][st] : mesh_of(w.loc_seg, w.loc_t_off, w.loc_n, t);
-            const int32_t t3 = 3 * __ldg(w.loc_t_off + j);
-            const int32_t ti3 = 3 * __ldg(w.loc_t_off + j + 1) - t3;
-            const int32_t h0 = __ldg(w.loc_h_off + j), hi = __ldg(w.loc_h_off + j + 1) - h0;
-            const int32_t v0 = __ldg(w.loc_v_off + j), vi = __ldg(w.loc_v_off + j + 1) - v0;
-            const int32_t g = h0 + (3 * t - t3);
-            const int32_t bo = HI + (h0 - t3) - ti3;
+            if (r < 0) row = mesh_row(w, mesh_of(w.loc_seg, w.loc_t_off, w.loc_n, t), HI);
+            const int32_t g = row.h0 + (3 * t - row.t3);
             int32_t o[3];
 #pragma unroll
             for (int k = 0; k < 3; k++) {
@@ -344,12 +361,29 @@ __global__ void __launch_bounds__(LE_THREADS) k_longest_edge_batch(MeshView m, W
             }
 #pragma unroll
             for (int k = 0; k < 3; k++) {
-                if ((uint32_t)o[k] >= (uint32_t)vi) { o[k] = 0; bad = true; }
-                if ((uint32_t)tw[q][k] >= (uint32_t)hi) { tw[q][k] = ti3; bad = true; }
-                tw[q][k] = tw[q][k] < ti3 ? t3 + tw[q][k] : bo + tw[q][k];
-                w.u_twin[3 * t + k] = tw[q][k];
-                p[q][k] = __ldg(m.xy + v0 + o[k]);
+                if ((uint32_t)o[k] >= (uint32_t)row.vi) { o[k] = 0; bad = true; }
+                if ((uint32_t)tw[q][k] >= (uint32_t)row.hi) { tw[q][k] = row.ti3; bad = true; }
+                tw[q][k] += tw[q][k] < row.ti3 ? row.t3 : row.bo;
+                p[q][k] = __ldg(m.xy + row.v0 + o[k]);
             }
+        }
+        // the union twins go out from the stage's own buffer, in whole 16-byte
+        // words (every lane has read its local ones)
+        __syncwarp();
+        int32_t *ut = s_tw[warp][st];
+#pragma unroll
+        for (int q = 0; q < PER; q++) {
+            const int32_t lt = lane + 32 * q;
+#pragma unroll
+            for (int k = 0; k < 3; k++) ut[3 * lt + k] = tw[q][k];
+        }
+        __syncwarp();
+        if (t0 + LE_TILE <= m.T) {
+#pragma unroll
+            for (int i = lane; i < 3 * LE_TILE / 4; i += 32)
+                reinterpret_cast<int4 *>(w.u_twin + 3 * (int64_t)t0)[i] = reinterpret_cast<const int4 *>(ut)[i];
+        } else {
+            for (int32_t i = lane; i < 3 * (m.T - t0); i += 32) w.u_twin[3 * (int64_t)t0 + i] = ut[i];
         }
 #pragma unroll
         for (int q = 0; q < PER; q++) {
@@ -662,23 +696,35 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_label_relink1(MeshView m, Wor
     const int32_t t = t0 + lane;
     const bool live = t < m.T;
     const int32_t e0 = 3 * t;
-    int32_t m0 = 0;  // batches: the mesh of the warp's first triangle
-    if (BATCH) {
-        if (lane == 0 && live) m0 = mesh_of(w.loc_seg, w.loc_t_off, w.loc_n, t0);
-        m0 = __shfl_sync(0xffffffffu, m0, 0);
-    }
     const int32_t ws = 3 * ((int32_t)threadIdx.x & ~31);  // the warp's first slot
     uint32_t F = 0, fl = 0;
     uint32_t kt = 3;          // the local index of the rotating half-edge (3: none)
     uint32_t kf = 3;          // that of the run's first half-edge (3: no frontier, or all of it)
     int32_t twk = 0;          // the rotating half-edge's twin (coming back to it finds a tip)
     uint32_t x = 0, lx = 0, ley = 0;  // the rotation: half-edge, its local index, its triangle's longest
+    uint32_t tw[3] = {0, 0, 0}, ltl = 0;
     if (live) {
-        uint32_t tw[3], ttri[3], tloc[3], lnb[3];
         tw[0] = (uint32_t)__ldg(m.twin + e0);
         tw[1] = (uint32_t)__ldg(m.twin + e0 + 1);
         tw[2] = (uint32_t)__ldg(m.twin + e0 + 2);
-        const uint32_t ltl = w.le[t];
+        ltl = w.le[t];
+    }
+    // batches: the mesh of the warp's first triangle (m0) and the thread's, its
+    // first union half-edge (sh), and from a union half-edge to its entry in the
+    // local arrays (gsh).  Most warps lie inside one mesh.
+    int32_t m0 = 0, sh = 0, gsh = 0;
+    bool one = true;
+    if (BATCH && t0 < m.T) {
+        m0 = mesh_of(w.loc_seg, w.loc_t_off, w.loc_n, t0);
+        int32_t mj = m0;
+        one = nE == 96 && eb + 96 <= 3 * __ldg(w.loc_t_off + m0 + 1);
+        if (!one && live)
+            while (mj + 1 < w.loc_n && __ldg(w.loc_t_off + mj + 1) <= t) mj++;
+        sh = 3 * __ldg(w.loc_t_off + mj);
+        gsh = __ldg(w.loc_h_off + mj) - sh;
+    }
+    if (live) {
+        uint32_t ttri[3], tloc[3], lnb[3];
         uint32_t twle = 0;
 #pragma unroll
         for (uint32_t k = 0; k < 3; k++) {
@@ -713,12 +759,6 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_label_relink1(MeshView m, Wor
         }
     }
     __syncwarp();  // every prev slot initialised before rotations write them
-    int32_t mj = 0, sh = 0;  // batches: the thread's mesh and its first union half-edge
-    if (BATCH && live) {
-        mj = m0;
-        while (mj + 1 < w.loc_n && __ldg(w.loc_t_off + mj + 1) <= t) mj++;
-        sh = 3 * __ldg(w.loc_t_off + mj);
-    }
     if (kt < 3u) {
         // while x is not frontier, x = CW(x).  The next step's twin is fetched
         // with this step's label.
@@ -744,7 +784,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_label_relink1(MeshView m, Wor
         const uint32_t dx = x - (uint32_t)eb;
         if (dx < 96u) s_pv[ws + (int32_t)dx] = e;  // (past the end of the mesh there is no x)
         else if (!BATCH) m.prev[x] = e;
-        else w.loc_prev[__ldg(w.loc_h_off + mj) + ((int32_t)x - sh)] = e - sh;  // e, x lie in mesh mj
+        else w.loc_prev[(int32_t)x + gsh] = e - sh;  // e and x lie in one mesh
         if ((int32_t)x == twk) add_tip(w, twk, steps);
     }
     __syncwarp();  // every prev slot is final
@@ -769,14 +809,19 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_label_relink1(MeshView m, Wor
     // each warp stores the links of its 96 half-edges in place, coalesced
     // (in a batch, also in the meshes' own indices and arrays; a batch's
     // union prev is never read, so it is not written)
-    if (!BATCH && nE == 96) {
+    if (nE == 96 && one) {
         if (lane < 24)
             reinterpret_cast<int4 *>(m.next + eb)[lane] = reinterpret_cast<const int4 *>(s_nx + ws)[lane];
-        int32_t *pd = m.prev + eb + lane;
-        const int32_t *ps = s_pv + ws + lane;
+        const int32_t *ps = s_pv + ws + lane, *ns = s_nx + ws + lane;
+        if (BATCH) {
+            int32_t *nd = w.loc_next + (eb + gsh) + lane;
+#pragma unroll
+            for (int i = 0; i < 96; i += 32) nd[i] = ns[i] - sh;
+        }
+        int32_t *pd = BATCH ? w.loc_prev + (eb + gsh) + lane : m.prev + eb + lane;
 #pragma unroll
         for (int i = 0; i < 96; i += 32)
-            if (ps[i] >= 0) pd[i] = ps[i];
+            if (ps[i] >= 0) pd[i] = ps[i] - sh;
         return;
     }
     int32_t bj = m0;
