@@ -255,18 +255,27 @@ __device__ __forceinline__ int32_t mesh_of(const int32_t *seg, const int32_t *t_
 // |v^| and |v^| <= |v|, by bit manipulation (no float64 instruction).  A
 // magnitude outside [2^-126, 2^61) (zero included) sets bad: the caller then
 // takes its exact float64 path.
-__device__ __forceinline__ float trunc_to_f32(double v, uint32_t &bad) {
-    uint32_t hi = (uint32_t)__double2hiint(v);
-    uint32_t lo = (uint32_t)__double2loint(v);
-    uint32_t mag = hi & 0x7FFFFFFFu;
+// trunc_to_f32_far leaves the test to the caller, once for several values: far
+// collects the largest distance of their exponents from the range's lower end,
+// and all lie inside it iff far < TRUNC_SPAN.
+constexpr uint32_t TRUNC_SPAN = (1084u - 897u) << 21;
+__device__ __forceinline__ float trunc_to_f32_far(double v, uint32_t &far) {
+    const uint32_t hi = (uint32_t)__double2hiint(v);
+    const uint32_t lo = (uint32_t)__double2loint(v);
     // biased float64 exponent must lie in [897, 1083]: |v| in [2^-126, 2^61)
-    bad |= (uint32_t)((mag - (897u << 20)) >= ((1084u - 897u) << 20));
+    // (doubling drops the sign)
+    far = max(far, 2u * hi - (897u << 21));
     // (hi:lo) << 3 puts the low 9 exponent bits at 31..23 and the top 23
     // significand bits at 22..0; subtracting 384 from that 9-bit field
     // rebiases 1023 -> 127 for exponents in range
-    uint32_t bits = __funnelshift_l(lo, hi, 3) - (384u << 23);
-    bits |= hi & 0x80000000u;
-    return __uint_as_float(bits);
+    const uint32_t bits = __funnelshift_l(lo, hi, 3) - (384u << 23);
+    return __uint_as_float(bits | (hi & 0x80000000u));
+}
+__device__ __forceinline__ float trunc_to_f32(double v, uint32_t &bad) {
+    uint32_t far = 0;
+    const float f = trunc_to_f32_far(v, far);
+    bad |= (uint32_t)(far >= TRUNC_SPAN);
+    return f;
 }
 
 // ---- implicit triangle layout (paper Section 4.2) -------------------------
