@@ -219,7 +219,9 @@ int polylla_generate_host(polylla_ctx *ctx, const polylla_host_mesh *in,
  * "poly_count", "tile_scan", "poly_list"), then "batch_meta" (the serving
  * loop's per-mesh metadata).
  * polylla_launch_count gives the number of kernels the last generate
- * launched (7 for a mesh or a batch, 8 for a served batch).
+ * launched (7 for a mesh or a batch, 8 for a served batch; 1 for a mesh of at
+ * most 2,048 triangles, unless stage times are on or polylla_set_tuning chose
+ * the launch settings of the seven).
  */
 int polylla_set_timing(polylla_ctx *ctx, int32_t enable);
 int polylla_get_stage_times(polylla_ctx *ctx, float *ms, int32_t n);

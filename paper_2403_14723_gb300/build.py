@@ -18,9 +18,10 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 SOURCES = ["polylla_api.cu", "kernels_label.cu", "kernels_repair.cu", "kernels_output.cu", "kernels_batch.cu",
-           "kernels_serve.cu", "polylla_noalloc.cu", "polylla_server.cu", "kernels_lepp.cu", "kernels_convex.cu"]
-HEADERS = [os.path.join(CSRC, "polylla_internal.cuh"), os.path.join(CSRC, "polylla_serve.cuh"),
-           os.path.join(CSRC, "serve_policy.h"), os.path.join(INCLUDE, "polylla.h")]
+           "kernels_serve.cu", "polylla_noalloc.cu", "polylla_server.cu", "kernels_lepp.cu", "kernels_convex.cu",
+           "kernels_small.cu"]
+HEADERS = [os.path.join(CSRC, "polylla_internal.cuh"), os.path.join(CSRC, "longest_edge.cuh"),
+           os.path.join(CSRC, "polylla_serve.cuh"), os.path.join(CSRC, "serve_policy.h"), os.path.join(INCLUDE, "polylla.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
               "--expt-relaxed-constexpr", "-I" + INCLUDE]
@@ -35,7 +36,8 @@ def nvcc_path() -> str:
 
 # the files that define the method's kernels (their DRAM traffic, recorded
 # from ncu, stays valid while these are unchanged)
-CORE_SOURCES = ["kernels_label.cu", "kernels_repair.cu", "kernels_output.cu", "polylla_internal.cuh"]
+CORE_SOURCES = ["kernels_label.cu", "kernels_repair.cu", "kernels_output.cu", "polylla_internal.cuh",
+                "longest_edge.cuh"]
 
 
 def core_digest() -> str:

@@ -42,6 +42,7 @@ struct polylla_ctx {
     cudaStream_t last_stream = nullptr;
     // batch: c->mesh is the union, bv the caller's local arrays
     bool is_batch = false;
+    bool staged = false;            // launch settings set by hand: the staged kernels on any size
     BatchView bv{};
     int32_t *poly_off = nullptr;    // [n+1] first polygon of each mesh
     int32_t *u_origin = nullptr, *u_twin = nullptr;  // union arrays, owned
@@ -262,7 +263,7 @@ static int alloc_work(polylla_ctx *c, const polylla_options *opt) {
     c->w.out_items = OUT_ITEMS_DEFAULT;
     c->w.rl_tile = RL_TILE_DEFAULT;
     c->w.rl_items = RL_ITEMS_DEFAULT;
-    if (polygons_configure() != 0 || relink_configure() != 0) return cuda_fail(c, cudaGetLastError());
+    if (polygons_configure() != 0 || relink_configure() != 0 || small_configure() != 0) return cuda_fail(c, cudaGetLastError());
     c->w.max_rot = (opt && opt->max_rotation > 0) ? opt->max_rotation : 4096;
     apply_cached_tuning(c);
     for (int i = 0; i < kStages; i++) {
@@ -426,6 +427,15 @@ int polylla_create_host(polylla_ctx **out, int32_t n_vertices, int32_t n_triangl
 // an event pair around every stage.
 static int enqueue(polylla_ctx *c, cudaStream_t s, bool timing) {
     for (int i = 0; i < kStages; i++) c->stage_ran[i] = false;
+    // small meshes: one kernel, unless stage times or events between the stages
+    // are asked for, or the stages' launch settings were set by hand
+    if (!c->is_batch && !timing && !c->staged && c->mesh.T <= SMALL_MAX && !c->wait_before_relink &&
+        !c->record_after_links) {
+        launch_small(c->mesh, c->w, s);
+        c->launches = 1;
+        CK(cudaGetLastError());
+        return POLYLLA_OK;
+    }
     auto begin = [&](int i) -> cudaError_t {
         c->stage_ran[i] = true;
         return timing ? cudaEventRecord(c->ev_begin[i], s) : cudaSuccess;
@@ -760,6 +770,7 @@ int polylla_set_tuning(polylla_ctx *c, const polylla_tuning *t) {
     if (!c || !t || !tuning_valid(c, *t)) return POLYLLA_ERR_INVALID_ARGUMENT;
     drop_graph(c);
     apply_tuning(c, *t);
+    c->staged = true;
     return POLYLLA_OK;
 }
 

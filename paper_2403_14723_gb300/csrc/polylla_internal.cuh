@@ -152,6 +152,9 @@ constexpr int LE_ITEMS_DEFAULT = 2;
 constexpr int RL_TILE_DEFAULT = 128;
 constexpr int RL_ITEMS_DEFAULT = 1;
 
+// meshes of up to so many triangles take one kernel of one block
+constexpr int SMALL_MAX = 2048;
+
 // bounded waits: iterations of an mbarrier try_wait loop before giving up
 constexpr int MBAR_WAIT_LIMIT = 1 << 22;
 
@@ -298,6 +301,9 @@ void launch_validate(const MeshView &m, int32_t *bad, cudaStream_t s);
 void launch_longest_edge(const MeshView &m, const Work &w, cudaStream_t s, bool chained);
 int longest_edge_blocks_per_sm(int32_t items);
 int longest_edge_batch_blocks_per_sm();
+// the whole generate of a single mesh of at most SMALL_MAX triangles (kernels_small.cu)
+void launch_small(const MeshView &m, const Work &w, cudaStream_t s);
+int small_configure();  // its shared memory on the current device; 0 on success
 void launch_label_relink(const MeshView &m, const Work &w, cudaStream_t s, bool chained);
 // allows the relink kernels their shared memory on the current device (once
 // per device before the first launch); 0 on success

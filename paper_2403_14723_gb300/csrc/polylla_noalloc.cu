@@ -65,7 +65,7 @@ static int device_setup(unsigned char **out, int *sms) {
         void *p = nullptr;
         int n = 0;
         if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return POLYLLA_ERR_CUDA;
-        if (polygons_configure() != 0 || relink_configure() != 0) return POLYLLA_ERR_CUDA;
+        if (polygons_configure() != 0 || relink_configure() != 0 || small_configure() != 0) return POLYLLA_ERR_CUDA;
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d) != cudaSuccess) return POLYLLA_ERR_CUDA;
         g_sms[d] = n > 0 ? n : 1;
         g_scratch_addr[d] = static_cast<unsigned char *>(p);
@@ -140,13 +140,17 @@ extern "C" int polylla_generate_noalloc(const polylla_mesh *mesh, int32_t *seeds
     // before it is read, so the previous call's contents never leak into
     // this one.
     cudaStream_t s = (cudaStream_t)stream;
-    launch_longest_edge(m, w, s, false);
-    launch_label_relink(m, w, s, true);
-    launch_chords(m, w, s, true);
-    launch_chord_links(m, w, s, true);
-    launch_poly_count(m, w, s, true);
-    launch_tile_scan(m, w, s, true);
-    launch_poly_list(m, w, s, true);
+    if (T <= SMALL_MAX) {
+        launch_small(m, w, s);
+    } else {
+        launch_longest_edge(m, w, s, false);
+        launch_label_relink(m, w, s, true);
+        launch_chords(m, w, s, true);
+        launch_chord_links(m, w, s, true);
+        launch_poly_count(m, w, s, true);
+        launch_tile_scan(m, w, s, true);
+        launch_poly_list(m, w, s, true);
+    }
     // status3 = {P, N_F, device error bits}, copied device to device
     if (cudaMemcpyAsync(status3, &w.ctrl->n_polygons, 2 * sizeof(int32_t), cudaMemcpyDeviceToDevice, s) !=
             cudaSuccess ||
