@@ -150,6 +150,16 @@ void polylla_destroy(polylla_ctx *ctx);
 const char *polylla_status_string(int status);
 
 /*
+ * polylla_dlpack: a DLPack descriptor (a DLManagedTensor of the DLPack ABI, as
+ * a "dltensor" capsule holds it) of n device integers at data, unsigned 8-bit
+ * (bits 8) or signed 32-bit (bits 32): how a caller's array library sees the
+ * arrays that this library owns without copying them.  It owns no device
+ * memory; its deleter frees the descriptor.  NULL for another width, n < 1,
+ * memory that is not a device's, or no host memory.
+ */
+void *polylla_dlpack(const void *data, int64_t n, int32_t bits);
+
+/*
  * Intermediate labels, for stage-by-stage checks (not needed to use the
  * output).  Device arrays owned by the context, valid after a generate
  * completes and until the next generate or destroy:

@@ -347,6 +347,46 @@ const char *polylla_status_string(int status) {
     }
 }
 
+// The part of the DLPack ABI (version 0.x, unversioned capsules) that a one-
+// dimensional integer array needs; the field order is the ABI's.
+namespace {
+struct DlTensor {
+    void *data;
+    int32_t device_type, device_id;  // 2: CUDA
+    int32_t ndim;
+    uint8_t code, bits;              // 0: signed, 1: unsigned integers
+    uint16_t lanes;
+    int64_t *shape, *strides;
+    uint64_t byte_offset;
+};
+struct DlManaged {
+    DlTensor t;
+    void *manager;
+    void (*deleter)(DlManaged *);
+    int64_t shape;                   // ours, past the ABI's fields
+};
+void dl_delete(DlManaged *m) { delete m; }
+}  // namespace
+
+void *polylla_dlpack(const void *data, int64_t n, int32_t bits) {
+    if (!data || n < 1 || (bits != 8 && bits != 32)) return nullptr;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, data) != cudaSuccess || at.type != cudaMemoryTypeDevice) return nullptr;
+    DlManaged *m = new (std::nothrow) DlManaged{};
+    if (!m) return nullptr;
+    m->shape = n;
+    m->t.data = const_cast<void *>(data);
+    m->t.device_type = 2;
+    m->t.device_id = at.device;
+    m->t.ndim = 1;
+    m->t.code = bits == 8 ? 1 : 0;
+    m->t.bits = (uint8_t)bits;
+    m->t.lanes = 1;
+    m->t.shape = &m->shape;
+    m->deleter = dl_delete;
+    return m;
+}
+
 int polylla_create(polylla_ctx **out, const polylla_mesh *mesh, const polylla_options *opt,
                    polylla_stream stream) {
     if (!out) return POLYLLA_ERR_INVALID_ARGUMENT;

@@ -135,6 +135,7 @@ _SIGNATURES = {
     "polylla_cuda_error": (ctypes.c_int, [ctypes.c_void_p]),
     "polylla_destroy": (None, [ctypes.c_void_p]),
     "polylla_status_string": (ctypes.c_char_p, [ctypes.c_int]),
+    "polylla_dlpack": (ctypes.c_void_p, [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32]),
     "polylla_get_labels": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(polylla_labels), ctypes.c_void_p]),
     "polylla_create_host": (ctypes.c_int, [ctypes.POINTER(ctypes.c_void_p), ctypes.c_int32, ctypes.c_int32,
                                            ctypes.c_int32, ctypes.POINTER(polylla_options)]),
@@ -209,8 +210,8 @@ def _check(rc: int, where: str):
 def _stream_ptr(stream):
     import torch
 
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:  # the current stream's handle, without a Stream object
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return ctypes.c_void_p(stream.cuda_stream)
 
 
@@ -224,21 +225,23 @@ def _dev_ptr(t, dtype, n):
     return ctypes.c_void_p(t.data_ptr())
 
 
-class _CudaArray:
-    """Zero-copy view of context-owned device memory for torch.as_tensor."""
-
-    def __init__(self, ptr: int, n: int, typestr: str):
-        self.__cuda_array_interface__ = {
-            "shape": (n,), "typestr": typestr, "data": (ptr, False), "version": 3, "strides": None,
-        }
+_new_capsule = ctypes.pythonapi.PyCapsule_New
+_new_capsule.restype = ctypes.py_object
+_new_capsule.argtypes = [ctypes.c_void_p, ctypes.c_char_p, ctypes.c_void_p]
 
 
-def _view(ptr, n, typestr, dtype):
+def _view(ptr, n, bits, dtype):
+    """Zero-copy tensor over n integers (int32 or uint8) of context-owned
+    device memory: a DLPack descriptor made by the library (a 2 us call; the
+    array interface took 5, and polygons() makes four)."""
     import torch
 
     if n == 0:
         return torch.empty(0, dtype=dtype, device="cuda")
-    return torch.as_tensor(_CudaArray(int(ptr), int(n), typestr), device="cuda")
+    t = load_library().polylla_dlpack(ctypes.c_void_p(ptr), n, bits)
+    if not t:
+        raise PolyllaError(-1, "polylla_dlpack")
+    return torch._C._from_dlpack(_new_capsule(t, b"dltensor", None))
 
 
 @dataclass
@@ -299,10 +302,10 @@ def polylla_get_polygons(ctx: int, stream=None) -> dict:
     P, NF = out.n_polygons, out.n_frontier
     return {
         "n_polygons": P, "n_frontier": NF,
-        "seeds": _view(out.seeds, P, "<i4", torch.int32),
-        "offsets": _view(out.offsets, P + 1, "<i4", torch.int32),
-        "he_list": _view(out.he_list, NF, "<i4", torch.int32),
-        "v_list": _view(out.v_list, NF, "<i4", torch.int32),
+        "seeds": _view(out.seeds, P, 32, torch.int32),
+        "offsets": _view(out.offsets, P + 1, 32, torch.int32),
+        "he_list": _view(out.he_list, NF, 32, torch.int32),
+        "v_list": _view(out.v_list, NF, 32, torch.int32),
     }
 
 
@@ -313,10 +316,10 @@ def polylla_get_labels(ctx: int, n_triangles: int, stream=None) -> dict:
     _check(load_library().polylla_get_labels(ctypes.c_void_p(ctx), ctypes.byref(out), _stream_ptr(stream)),
            "polylla_get_labels")
     return {
-        "longest_local": _view(out.longest_local, n_triangles, "|u1", torch.uint8),
-        "flags": _view(out.flags, n_triangles, "|u1", torch.uint8),
-        "tips": _view(out.tips, out.n_tips, "<i4", torch.int32),
-        "chords": _view(out.chords, out.n_tips, "<i4", torch.int32),
+        "longest_local": _view(out.longest_local, n_triangles, 8, torch.uint8),
+        "flags": _view(out.flags, n_triangles, 8, torch.uint8),
+        "tips": _view(out.tips, out.n_tips, 32, torch.int32),
+        "chords": _view(out.chords, out.n_tips, 32, torch.int32),
         "n_tips": out.n_tips,
     }
 
@@ -508,7 +511,7 @@ def polylla_batch_polygon_offsets(ctx: int, n_meshes: int):
     p = ctypes.c_void_p()
     _check(load_library().polylla_batch_polygon_offsets(ctypes.c_void_p(ctx), ctypes.byref(p)),
            "polylla_batch_polygon_offsets")
-    return _view(p.value, n_meshes + 1, "<i4", torch.int32)
+    return _view(p.value, n_meshes + 1, 32, torch.int32)
 
 
 def polylla_convexify(ctx: int, stream=None) -> None:
@@ -528,7 +531,7 @@ def polylla_convex_chords(ctx: int, stream=None):
                                                 _stream_ptr(stream)), "polylla_convex_chords")
     if n.value == 0:
         return torch.empty(0, dtype=torch.int32, device="cuda")
-    return _view(p.value, n.value, "<i4", torch.int32)
+    return _view(p.value, n.value, 32, torch.int32)
 
 
 def polylla_lepp_terminal(ctx: int, n_triangles: int, with_length: bool = True, stream=None):
