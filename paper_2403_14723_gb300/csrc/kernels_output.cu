@@ -727,6 +727,19 @@ __global__ void __launch_bounds__(TILE / IPT, TILE == 1024 && IPT == 4 ? 6 : 1) 
     }
 }
 
+// The control block into pinned host memory.  A kernel's store and not a copy:
+// copies of one direction go through one engine in order, so the 32-byte copy of
+// polylla_generate_host waited behind the links on their way out (0.5 M triangles:
+// 272 us a call, 264 with the store); after a generate alone it took 2 us longer.
+__global__ void k_ctrl_out(const int32_t *ctrl, int32_t *host) {
+    if (threadIdx.x < sizeof(DevCtrl) / sizeof(int32_t)) host[threadIdx.x] = ctrl[threadIdx.x];
+}
+
+cudaError_t launch_ctrl_out(const Work &w, DevCtrl *host, cudaStream_t s) {
+    return launch_kernel(k_ctrl_out, 1, 32, 0, s, false, reinterpret_cast<const int32_t *>(w.ctrl),
+                         reinterpret_cast<int32_t *>(host));
+}
+
 // ---- launch configurations (tile triangles, triangles per thread) ------------
 template <int TILE, int IPT>
 constexpr size_t count_smem() {

@@ -562,7 +562,7 @@ static int device_status(const DevCtrl &h) {
 }
 
 static int read_ctrl(polylla_ctx *c, cudaStream_t s) {
-    CK(cudaMemcpyAsync(c->h_ctrl, c->w.ctrl, sizeof(DevCtrl), cudaMemcpyDeviceToHost, s));
+    CK(launch_ctrl_out(c->w, c->h_ctrl, s));
     CK(cudaStreamSynchronize(s));
     return POLYLLA_OK;
 }

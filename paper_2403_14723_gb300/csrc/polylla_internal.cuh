@@ -171,7 +171,7 @@ __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.laun
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // chained only directly behind a kernel of the chain on the same stream
 template <typename... P, typename... A>
-void launch_kernel(void (*kernel)(P...), int64_t blocks, int threads, size_t smem, cudaStream_t s, bool chained,
+cudaError_t launch_kernel(void (*kernel)(P...), int64_t blocks, int threads, size_t smem, cudaStream_t s, bool chained,
                    const A &...args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)blocks);
@@ -183,7 +183,7 @@ void launch_kernel(void (*kernel)(P...), int64_t blocks, int threads, size_t sme
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = chained ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // an error stays pending for the caller's check
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // an error also stays pending
 }
 
 // ---- bulk copies (TMA engine) and mbarriers, inline PTX --------------------
@@ -328,6 +328,7 @@ void launch_poly_list(const MeshView &m, const Work &w, cudaStream_t s, bool cha
 int polygons_configure();
 bool polygons_config_valid(int32_t tile, int32_t items);
 int polygons_blocks_per_sm(int32_t tile, int32_t items);
+cudaError_t launch_ctrl_out(const Work &w, DevCtrl *host, cudaStream_t s);  // host: pinned
 // exclusive scan of n u64 values by one block; *grand gets the sum
 void launch_scan_u64(const unsigned long long *in, unsigned long long *out, int32_t n, unsigned long long *grand,
                      cudaStream_t s);
