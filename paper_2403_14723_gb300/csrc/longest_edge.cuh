@@ -40,33 +40,20 @@ __device__ __forceinline__ double sq_len_f64(double2 a, double2 b) {
     return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
 }
 
-// The exact float64 argmax; tw0..tw2 are the twins of e0, e0 + 1, e0 + 2 (equal
-// lengths go to the smaller edge id min(e, twin e)).  out is an edge known to be
-// shorter (3: none): its length is left out, since float64 is what this path
-// spends its time on.
-static __device__ __noinline__ uint32_t longest_exact(double2 p0, double2 p1, double2 p2, int32_t e0, int32_t tw0,
-                                               int32_t tw1, int32_t tw2, uint32_t out) {
+// The edges of the largest float64 length, a bit each (several: a tie).  out is an
+// edge known to be shorter (3: none): its length is left out, since float64 is what
+// this path spends its time on.
+static __device__ __noinline__ uint32_t longest_exact(double2 p0, double2 p1, double2 p2, uint32_t out) {
     // from the vertex after it on: edges a, b and (perhaps out) c
-    const uint32_t a = out == 0u ? 1u : (out == 1u ? 2u : 0u), b = a == 2u ? 0u : a + 1u, c = b == 2u ? 0u : b + 1u;
+    const uint32_t a = out == 0u ? 1u : (out == 1u ? 2u : 0u), b = a == 2u ? 0u : a + 1u;
     const double2 pa = a == 0u ? p0 : (a == 1u ? p1 : p2);
     const double2 pb = a == 0u ? p1 : (a == 1u ? p2 : p0);
     const double2 pc = a == 0u ? p2 : (a == 1u ? p0 : p1);
-    const int32_t twa = a == 0u ? tw0 : (a == 1u ? tw1 : tw2);
-    const int32_t twb = a == 0u ? tw1 : (a == 1u ? tw2 : tw0);
-    uint32_t best = a;
-    double d = sq_len_f64(pa, pb);
-    int32_t id = min(e0 + (int32_t)a, twa);
-    const double db = sq_len_f64(pb, pc);
-    const int32_t idb = min(e0 + (int32_t)b, twb);
-    if (db > d || (db == d && idb < id)) {
-        best = b;
-        d = db;
-        id = idb;
-    }
-    if (out > 2u) {
-        const double dc = sq_len_f64(pc, pa);
-        const int32_t idc = min(e0 + (int32_t)c, tw2);  // a is 0, c is 2
-        if (dc > d || (dc == d && idc < id)) best = c;
+    const double da = sq_len_f64(pa, pb), db = sq_len_f64(pb, pc);
+    uint32_t best = (db > da ? 0u : 1u << a) | (db >= da ? 1u << b : 0u);
+    if (out > 2u) {  // a is 0, b is 1, c is 2
+        const double dc = sq_len_f64(pc, pa), d = db > da ? db : da;
+        best = (dc > d ? 0u : best) | (dc >= d ? 4u : 0u);
     }
     return best;
 }
@@ -101,7 +88,22 @@ __device__ __forceinline__ uint32_t longest_of(double2 p0, double2 p1, double2 p
         const float least = fminf(lo01, d2);
         uint32_t out = least == d2 ? 2u : (least == d0 ? 0u : 1u);
         if (!(far < TRUNC_SPAN && __fsub_rn(dm, least) > b2)) out = 3u;
-        k = longest_exact(p0, p1, p2, e0, tw(0), tw(1), tw(2), out);
+        // equal lengths go to the smaller edge id min(e, twin e).  Only they read
+        // the twins: every triangle of this path waited for three loads from memory.
+        const uint32_t ties = longest_exact(p0, p1, p2, out);
+        k = ties >> 1;  // of one bit: 1, 2 or 4
+        if (ties & (ties - 1u)) {
+            int32_t least_id = INT32_MAX;
+#pragma unroll
+            for (int j = 0; j < 3; j++) {
+                if (!((ties >> j) & 1u)) continue;
+                const int32_t id = min(e0 + j, tw(j));
+                if (id < least_id) {
+                    least_id = id;
+                    k = (uint32_t)j;
+                }
+            }
+        }
     }
     return k;
 }
