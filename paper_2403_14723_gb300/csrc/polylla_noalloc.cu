@@ -75,6 +75,18 @@ static int device_setup(unsigned char **out, int *sms) {
     return POLYLLA_OK;
 }
 
+// status3 = {P, N_F, device error bits}: one chained launch, where two copies on
+// the device waited for their turn one after the other (130 k triangles, a call:
+// 69.1 -> 62.4 us)
+static __global__ void k_noalloc_status(const DevCtrl *c, int32_t *status3) {
+    chain_wait();
+    if (threadIdx.x == 0) {
+        status3[0] = c->n_polygons;
+        status3[1] = c->n_frontier;
+        status3[2] = c->error;
+    }
+}
+
 extern "C" int polylla_generate_noalloc(const polylla_mesh *mesh, int32_t *seeds, int32_t *offsets,
                                         int32_t *he_list, int32_t *v_list, int32_t *status3,
                                         polylla_stream stream) {
@@ -151,11 +163,7 @@ extern "C" int polylla_generate_noalloc(const polylla_mesh *mesh, int32_t *seeds
         launch_tile_scan(m, w, s, true);
         launch_poly_list(m, w, s, true);
     }
-    // status3 = {P, N_F, device error bits}, copied device to device
-    if (cudaMemcpyAsync(status3, &w.ctrl->n_polygons, 2 * sizeof(int32_t), cudaMemcpyDeviceToDevice, s) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(status3 + 2, &w.ctrl->error, sizeof(int32_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return POLYLLA_ERR_CUDA;
+    launch_kernel(k_noalloc_status, 1, 32, 0, s, true, static_cast<const DevCtrl *>(w.ctrl), status3);
     if (cudaGetLastError() != cudaSuccess) return POLYLLA_ERR_CUDA;
     return POLYLLA_OK;
 }
