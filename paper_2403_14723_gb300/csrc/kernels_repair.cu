@@ -56,8 +56,8 @@ __global__ void __launch_bounds__(256) k_chords(MeshView m, Work w) {
 
 // Blocks of a kernel over a list of unknown length: one per `per` triangles (a
 // list longer than that takes the kernel's loop more often), at most the chip
-// full.  608 blocks for whatever mesh cost the smallest ones their launch, and
-// the links of 500 k chords three rounds.
+// full.  608 blocks were too many for a small mesh (8 us a launch for nothing) and
+// too few for a convexification's chords (several rounds of chains).
 static int list_blocks(const MeshView &m, const Work &w, int32_t per) {
     const int64_t want = m.T / per + 1, most = 2 * (int64_t)w.persistent_blocks;
     return (int)(want < most ? want : most);
