@@ -301,7 +301,10 @@ __global__ void __launch_bounds__(LE_THREADS, PER == 2 ? 4 : 2) k_longest_edge_b
             if (t < m.T)
                 w.le[t] = (uint8_t)longest_of(p[q][0], p[q][1], p[q][2], 3 * t, [twq](int k) { return twq[k]; });
         }
-        __syncwarp();  // stage st is refilled next iteration
+        // stage st is refilled next iteration: every lane's writes of its twins come
+        // before the copy engine's
+        fence_proxy_async_smem();
+        __syncwarp();
     }
     if (bad) atomicOr(w.input_err, 1);
 }
