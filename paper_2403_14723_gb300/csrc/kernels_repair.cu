@@ -33,20 +33,26 @@ __device__ __forceinline__ void set_start(uint8_t *flags, int32_t e) { set_flag_
 __global__ void __launch_bounds__(256) k_chords(MeshView m, Work w) {
     chain_next();
     chain_wait();
+    const int32_t HI = 3 * m.T;
     int32_t n = w.ctrl->n_tips;
     if (n > w.tip_cap) n = w.tip_cap;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int32_t d = w.chords[i];
         int32_t y = w.tips[i];
         int32_t ty = __ldg(m.twin + y);
-        if (d > w.max_rot) {
+        // around a tip every edge is interior.  A mesh that was not validated can
+        // have a border twin here: the links of the border are not the layout's
+        // (and a batch's union holds none), so the walk ends with an error.
+        bool ok = d <= w.max_rot && ty < HI;
+        for (int32_t s = 0; ok && s < (d - 1) / 2 + 1; s++) {
+            y = nx_of(ty);
+            ty = __ldg(m.twin + y);
+            ok = ty < HI;
+        }
+        if (!ok) {
             atomicOr(&w.ctrl->error, DEV_ERR_NONTERMINATING);
             w.chords[i] = -1;
             continue;
-        }
-        for (int32_t s = 0; s < (d - 1) / 2 + 1; s++) {
-            y = nx_of(ty);
-            ty = __ldg(m.twin + y);
         }
         w.chords[i] = y;
         set_f1(w.flags, y);
