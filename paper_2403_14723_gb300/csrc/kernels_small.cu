@@ -97,15 +97,19 @@ __global__ void __launch_bounds__(SM_THREADS) k_small(MeshView m, Work w) {
             err |= DEV_ERR_CAPACITY;
             continue;
         }
-        int32_t y = f;
-        if (d > w.max_rot) {
-            err |= DEV_ERR_NONTERMINATING;
-            y = -1;
-        } else {
-            for (int32_t r = 0; r < (d - 1) / 2 + 1; r++) y = nx_of(s_tw[y]);
-            const int32_t ty = s_tw[y];
+        int32_t y = f, ty = s_tw[f];
+        bool ok = d <= w.max_rot && ty < HI;  // a border twin: not a valid mesh (as in k_chords)
+        for (int32_t r = 0; ok && r < (d - 1) / 2 + 1; r++) {
+            y = nx_of(ty);
+            ty = s_tw[y];
+            ok = ty < HI;
+        }
+        if (ok) {
             atomicOr(s_fl + tri_of(y), 1u << loc_of(y));
             atomicOr(s_fl + tri_of(ty), 1u << loc_of(ty));
+        } else {
+            err |= DEV_ERR_NONTERMINATING;
+            y = -1;
         }
         w.tips[slot] = f;
         w.chords[slot] = y;

@@ -104,3 +104,22 @@ def test_served_tip_with_a_border_twin(pinned):
         info = srv.wait(srv.submit(hr))
         assert info["status"] == 0
         assert np.array_equal(hr.result(info)["next"], r.next_out)
+
+
+@pytest.mark.parametrize("which", [0, 4, -1])
+@pytest.mark.parametrize("kind", [2, 3])
+def test_small_mesh_tip_with_a_border_twin(kind, which):
+    build.build_library()
+    mesh, r = _tip_mesh()
+    dm = polylla.DeviceMesh.from_host(mesh)
+    value, status = _bad_twins(mesh)[kind]
+    bad = int(r.tip_out[which])
+    with polylla.Polylla(dm, validate=False) as p:
+        dm.twin[bad] = value
+        p.generate()
+        assert polylla.polylla_launch_count(p.ctx) == 1
+        _expect(*_labels_of_failed_run(p.ctx, status), r, 0, bad)
+        dm.twin[bad] = int(mesh.twin[bad])
+        p.generate()
+        p.polygons()
+        assert np.array_equal(dm.next.cpu().numpy(), r.next_out) and np.array_equal(dm.prev.cpu().numpy(), r.prev_out)
