@@ -207,10 +207,10 @@ __global__ void k_batch_meta(BatchView b, const int32_t *offsets, const int32_t 
         int32_t lo = 0, hi = n - 1;
         while (lo < hi) {
             const int32_t mid = (lo + hi + 1) >> 1;
-            if (__ldg(poly_off + mid) + mid <= q) lo = mid;
+            if (poly_off[mid] + mid <= q) lo = mid;
             else hi = mid - 1;
         }
-        const int32_t p0 = __ldg(poly_off + lo);
+        const int32_t p0 = poly_off[lo];
         local_offsets[q] = offsets[p0 + (q - p0 - lo)] - offsets[p0];
     }
 }

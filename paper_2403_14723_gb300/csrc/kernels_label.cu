@@ -376,6 +376,13 @@ void launch_longest_edge(const MeshView &m, const Work &w, cudaStream_t s, bool 
 // slower: on row-major grids half of each vertex fan lies in the next row,
 // outside any tile narrower than a row.)
 // ===========================================================================
+// the twin of interior half-edge e: a batch's union twins are written by the
+// kernel before this one, a mesh's own are the caller's input (see chain_wait)
+template <bool BATCH, typename I>
+__device__ __forceinline__ int32_t twin_of(const MeshView &m, I e) {
+    return BATCH ? ld_chain(m.twin + e) : __ldg(m.twin + e);
+}
+
 __device__ __forceinline__ int32_t div3(int32_t x) { return (int32_t)((uint32_t)x / 3u); }
 
 // A rotation came back to its tip's only frontier half-edge f, steps steps past
@@ -423,9 +430,9 @@ __global__ void __launch_bounds__(NT, 2048 / NT / IPT) k_label_relink(MeshView m
         int32_t tw[3], ttri[3];
         uint32_t tloc[3], lnb[3];
         if (live) {
-            tw[0] = __ldg(m.twin + e0);
-            tw[1] = __ldg(m.twin + e0 + 1);
-            tw[2] = __ldg(m.twin + e0 + 2);
+            tw[0] = twin_of<BATCH>(m, e0);
+            tw[1] = twin_of<BATCH>(m, e0 + 1);
+            tw[2] = twin_of<BATCH>(m, e0 + 2);
             const uint32_t ltl = w.le[t];
             uint32_t F = 0, twle = 0;
 #pragma unroll
@@ -480,7 +487,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT / IPT) k_label_relink(MeshView m
         uint32_t ley = ((uint32_t)tk.w >> 2) & 3u;
         uint32_t lx = ly == 2u ? 0u : ly + 1u;
         int32_t x = 3 * ty + (int32_t)lx;
-        int32_t tx = __ldg(m.twin + x);
+        int32_t tx = twin_of<BATCH>(m, x);
         int32_t steps = 0;
         while (true) {
             if (tx >= HI) break;                     // border edge: frontier
@@ -489,7 +496,7 @@ __global__ void __launch_bounds__(NT, 2048 / NT / IPT) k_label_relink(MeshView m
             const uint32_t lxn = ltx == 2u ? 0u : ltx + 1u;
             const int32_t xn = 3 * ttx + (int32_t)lxn;
             const uint32_t lex = w.le[ttx];
-            const int32_t txn = __ldg(m.twin + xn);
+            const int32_t txn = twin_of<BATCH>(m, xn);
             if (ley != lx && lex != ltx) break;      // neither half longest: frontier
             ley = lex;
             x = xn;
@@ -616,9 +623,9 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_label_relink1(MeshView m, Wor
     uint32_t x = 0, lx = 0, ley = 0;  // the rotation: half-edge, its local index, its triangle's longest
     uint32_t tw[3] = {0, 0, 0}, ltl = 0;
     if (live) {
-        tw[0] = (uint32_t)__ldg(m.twin + e0);
-        tw[1] = (uint32_t)__ldg(m.twin + e0 + 1);
-        tw[2] = (uint32_t)__ldg(m.twin + e0 + 2);
+        tw[0] = (uint32_t)twin_of<BATCH>(m, e0);
+        tw[1] = (uint32_t)twin_of<BATCH>(m, e0 + 1);
+        tw[2] = (uint32_t)twin_of<BATCH>(m, e0 + 2);
         ltl = w.le[t];
     }
     // batches (looked up while the twins are on their way; with the fast stores
@@ -677,14 +684,14 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_label_relink1(MeshView m, Wor
         // while x is not frontier, x = CW(x).  The next step's twin is fetched
         // with this step's label.
         const int32_t e = e0 + (int32_t)kt;
-        uint32_t tx = (uint32_t)__ldg(m.twin + x);
+        uint32_t tx = (uint32_t)twin_of<BATCH>(m, x);
         int32_t steps = 0;
         while (tx < HI) {                            // a border edge is frontier
             const uint32_t ttx = tx / 3u;
             const uint32_t ltx = tx - 3u * ttx;
             const uint32_t xn = ltx == 2u ? tx - 2u : tx + 1u;
             const uint32_t lex = w.le[ttx];
-            const uint32_t txn = (uint32_t)__ldg(m.twin + xn);
+            const uint32_t txn = (uint32_t)twin_of<BATCH>(m, xn);
             if (ley != lx && lex != ltx) break;      // neither half longest: frontier
             ley = lex;
             x = xn;

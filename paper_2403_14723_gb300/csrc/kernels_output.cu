@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(TILE / (2 * IPT)) k_poly_count(MeshView m, Wor
             } else if (out) {
                 while (x > e) {
                     const uint32_t d = (uint32_t)(x - eb);
-                    x = d < ne ? s_nx[d] : __ldg(m.next + x);
+                    x = d < ne ? s_nx[d] : ld_chain(m.next + x);
                     if (++L > HI) {
                         runaway = true;
                         x = -1;
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(TILE / (2 * IPT)) k_poly_count(MeshView m, Wor
             // waits for its slowest lane, which is outside the tile
             int32_t j = 0;
             do {
-                const int32_t y = __ldg(m.next + x);
+                const int32_t y = ld_chain(m.next + x);
                 if (held) p[j] = x;
                 x = y;
             } while (++j < XCHUNK && x > e);
@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(TILE / IPT, TILE == 1024 && IPT == 4 ? 6 : 1) 
         for (; k > 0; k--, pos++) {
             emit(pos, x, she, sb);
             const uint32_t d = (uint32_t)(x - eb);
-            x = d < ne ? s_nx[d] : __ldg(m.next + x);
+            x = d < ne ? s_nx[d] : ld_chain(m.next + x);
         }
     };
     auto mesh_shift = [&](int32_t j, int32_t &she, int32_t &sb) {
@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(TILE / IPT, TILE == 1024 && IPT == 4 ? 6 : 1) 
             int32_t y = x;
             k = 0;
             do {
-                y = __ldg(m.next + y);
+                y = ld_chain(m.next + y);
                 k++;
             } while (y != x && k < HI);
         }
@@ -663,7 +663,7 @@ __global__ void __launch_bounds__(TILE / IPT, TILE == 1024 && IPT == 4 ? 6 : 1) 
         for (int j = 0; j < 4; j++) {
             const uint32_t q = q0 + 2 * j + (lane >> 4);
             c[j] = q < ncross ? cross[q] : make_int4(0, 0, 0, 0);
-            h[j] = c[j].x < 0 ? __ldg(w.cross_pool + 16 * (int64_t)(cown - c[j].x) + hl) : 0;
+            h[j] = c[j].x < 0 ? ld_chain(w.cross_pool + 16 * (int64_t)(cown - c[j].x) + hl) : 0;
         }
 #pragma unroll
         for (int j = 0; j < 4; j++) {
@@ -675,7 +675,7 @@ __global__ void __launch_bounds__(TILE / IPT, TILE == 1024 && IPT == 4 ? 6 : 1) 
                 k -= XCHUNK;
                 if (k <= 0) break;
                 pos += XCHUNK;
-                y = __ldg(w.cross_pool + 16 * (int64_t)__shfl_sync(hmask, y, 15, 16) + hl);
+                y = ld_chain(w.cross_pool + 16 * (int64_t)__shfl_sync(hmask, y, 15, 16) + hl);
             }
         }
     }

@@ -6,7 +6,7 @@
 
 namespace polylla {
 
-__device__ __forceinline__ bool f1_of(const uint8_t *__restrict__ flags, int32_t e, int32_t HI) {
+__device__ __forceinline__ bool f1_of(const uint8_t *flags, int32_t e, int32_t HI) {
     if (e >= HI) return true;  // border half-edges are always frontier
     return (flags[tri_of(e)] >> loc_of(e)) & 1u;
 }
@@ -39,14 +39,14 @@ __global__ void __launch_bounds__(256) k_chords(MeshView m, Work w) {
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int32_t d = w.chords[i];
         int32_t y = w.tips[i];
-        int32_t ty = __ldg(m.twin + y);
+        int32_t ty = ld_chain(m.twin + y);
         // around a tip every edge is interior.  A mesh that was not validated can
         // have a border twin here: the links of the border are not the layout's
         // (and a batch's union holds none), so the walk ends with an error.
         bool ok = d <= w.max_rot && ty < HI;
         for (int32_t s = 0; ok && s < (d - 1) / 2 + 1; s++) {
             y = nx_of(ty);
-            ty = __ldg(m.twin + y);
+            ty = ld_chain(m.twin + y);
             ok = ty < HI;
         }
         if (!ok) {
@@ -115,7 +115,7 @@ __device__ __forceinline__ void relink_around(const MeshView &m, const Work &w, 
         a = tc;
         b = nx_of(tc);
         while (true) {
-            const int32_t tb = __ldg(m.twin + b);
+            const int32_t tb = ld_chain(m.twin + b);
             if (f1_of(w.flags, b, HI)) break;
             b = nx_of(tb);
             if (++steps > w.max_rot) { atomicOr(&w.ctrl->error, DEV_ERR_NONTERMINATING); return; }
@@ -125,10 +125,10 @@ __device__ __forceinline__ void relink_around(const MeshView &m, const Work &w, 
         // interior half-edge before it, a, is twin(z)
         b = c;
         a = pv_of(c);
-        int32_t z = __ldg(m.twin + a);
+        int32_t z = ld_chain(m.twin + a);
         while (z < HI) {
             const int32_t pz = pv_of(z);
-            const int32_t nz = __ldg(m.twin + pz);
+            const int32_t nz = ld_chain(m.twin + pz);
             if (f1_of(w.flags, z, HI)) break;
             a = pz;
             z = nz;
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(256) k_chord_links(MeshView m, Work w, const i
         const int64_t q = cw ? i : i - 2 * (int64_t)n;
         const int32_t c0 = list[q >> 1];
         if (c0 < 0) continue;
-        const int32_t t0 = __ldg(m.twin + c0);
+        const int32_t t0 = ld_chain(m.twin + c0);
         relink_around(m, w, q & 1 ? t0 : c0, q & 1 ? c0 : t0, cw, HI);
     }
 }

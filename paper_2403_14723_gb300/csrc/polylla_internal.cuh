@@ -169,8 +169,22 @@ constexpr int MBAR_WAIT_LIMIT = 1 << 22;
 // after all kernels before it; without a chained launch both are no-ops.  A pass of
 // 4 k triangles 87.8 -> 76.6 us, of 2 M 155.7 -> 146.6, of the 4096 grid 1,116 ->
 // 1,110.
+// A chained kernel is resident while the kernels before it still write, so only
+// what no kernel of its chain writes may be read through the read-only path
+// (__ldg, const __restrict__): the caller's mesh arrays (coords, origin, twin) and
+// a batch's tables.  next, prev, labels, flags, lists, records, the chunk pool,
+// polygon ranges and a batch's union twins take ordinary loads.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// an ordinary load of what an earlier kernel of the chain wrote and this one does not
+// write, behind chain_wait (volatile keeps it there; without the compiler's aliasing
+// rules it takes no more registers than __ldg: written as m.next[x] the listing
+// spilled, and the 4096 grid took 1,058 us against 1,052)
+__device__ __forceinline__ int32_t ld_chain(const int32_t *p) {
+    int32_t v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 // chained only directly behind a kernel of the chain on the same stream
 template <typename... P, typename... A>
 cudaError_t launch_kernel(void (*kernel)(P...), int64_t blocks, int threads, size_t smem, cudaStream_t s, bool chained,
