@@ -228,8 +228,10 @@ static int alloc_work(polylla_ctx *c, const polylla_options *opt) {
     c->w.poly_wtot = (unsigned long long *)p;
     c->w.cross_own = (int32_t)cross_own_count(T);
     c->w.cross_more = (int32_t)cross_more_count(T);
-    if ((rc = dev_alloc(c, &p, 64 * (size_t)(cross_own_count(T) + cross_more_count(T))))) return rc;
-    c->w.cross_pool = (int32_t *)p;
+    if (!c->is_batch) {  // (a batch's: batch_alloc)
+        if ((rc = dev_alloc(c, &p, (size_t)cross_bytes(T)))) return rc;
+        c->w.cross_pool = (int32_t *)p;
+    }
     if ((rc = dev_alloc(c, &p, sizeof(int32_t) * (size_t)T))) return rc;
     c->w.seeds = (int32_t *)p;
     if ((rc = dev_alloc(c, &p, sizeof(int32_t) * (size_t)(T + 1)))) return rc;
@@ -298,10 +300,15 @@ static int batch_alloc(polylla_ctx *c, int32_t n, int32_t V, int32_t T, int32_t 
     for (int k = 0; k < 4 && !rc; k++)
         if ((rc = dev_alloc(c, &p, sizeof(int32_t) * (size_t)(n + 1))) == 0) d_off[k] = (int32_t *)p;
     if (!rc && (rc = dev_alloc(c, &p, sizeof(int32_t) * (size_t)(n + 1))) == 0) c->poly_off = (int32_t *)p;
-    if (!rc && (rc = dev_alloc(c, &p, 4 * (size_t)H)) == 0) c->u_origin = (int32_t *)p;
+    // the union origin and prev serve the layout check at create, and no kernel of a
+    // generate: the crossing walks' pool has their memory from then on
+    if (!rc && (rc = dev_alloc(c, &p, (size_t)union_block(T, H))) == 0) {
+        c->u_origin = (int32_t *)p;
+        c->mesh.prev = (int32_t *)((char *)p + union_part(H));
+        c->w.cross_pool = (int32_t *)p;
+    }
     if (!rc && (rc = dev_alloc(c, &p, 4 * (size_t)H)) == 0) c->u_twin = (int32_t *)p;
     if (!rc && (rc = dev_alloc(c, &p, 4 * (size_t)H)) == 0) c->mesh.next = (int32_t *)p;
-    if (!rc && (rc = dev_alloc(c, &p, 4 * (size_t)H)) == 0) c->mesh.prev = (int32_t *)p;
     if (!rc && (rc = dev_alloc(c, &p, sizeof(int32_t) * (size_t)seg_count(T))) == 0) c->w.loc_seg = (int32_t *)p;
     if (!rc && (rc = dev_alloc(c, &p, sizeof(int32_t))) == 0) c->w.input_err = (int32_t *)p;
     if (!rc && cudaMemset(c->w.input_err, 0, sizeof(int32_t)) != cudaSuccess) rc = POLYLLA_ERR_CUDA;

@@ -15,12 +15,13 @@
 //   poly_rec [T] u32     per polygon, at its output warp's first triangle on:
 //                        its minimum within the warp's half-edges, its length
 //                        and its chunk of the pool
-//   cross_pool [T/8+T/32+512][16] i32  the half-edges that a polygon which
-//                        leaves its tile visits from there on
+//   cross_pool [cross_own_count(T) + cross_more_count(T)][16] i32  the half-edges that a polygon which
+//                        leaves its tile visits from there on (in a batch, in
+//                        the memory of the union origin and prev)
 //   poly_wtot [T/64+66] u64  per output warp: its (polygons, length) total
 //   seeds [T], offsets [T+1], he_list [3T], v_list [3T]   CSR output
 //   ctrl          DevCtrl       counters and the device error word
-// A batch context adds the union origin/twin/next/prev [H] (origin and the
+// A batch context adds the union origin/twin/next/prev [H] (origin, prev and the
 // border entries of twin are only filled by the layout check at create; every
 // generate writes the interior twin entries from the meshes' own arrays), the
 // per-mesh prefix sums and polygon ranges, and the input-check word.
@@ -138,8 +139,16 @@ __host__ __device__ constexpr int64_t out_warp_count(int64_t T) { return (T + OU
 // grids, 0.02 on Delaunay meshes; the walks that find no chunk cost the
 // listing kernel a chain of loads), then those for long walks
 constexpr int XQUOTA = 8;
-__host__ __device__ constexpr int64_t cross_own_count(int64_t T) { return (T + OUT_TILE_MAX) / XQUOTA; }
-__host__ __device__ constexpr int64_t cross_more_count(int64_t T) { return T / 32 + 256; }
+// (a tile's walks use at most 255 chunks, and at most one per triangle)
+__host__ __device__ constexpr int64_t cross_own_count(int64_t T) { return T / XQUOTA + (T < 256 ? T : 256); }
+__host__ __device__ constexpr int64_t cross_more_count(int64_t T) { return T / 32 + (T < 2048 ? T / 8 : 256); }
+__host__ __device__ constexpr int64_t cross_bytes(int64_t T) { return 64 * (cross_own_count(T) + cross_more_count(T)); }
+// A batch has the pool in the memory of its union origin and prev, which only the
+// layout check at create uses: bytes of that block, and of each array's part
+__host__ __device__ constexpr int64_t union_part(int64_t H) { return (4 * H + 255) / 256 * 256; }
+__host__ __device__ constexpr int64_t union_block(int64_t T, int64_t H) {
+    return union_part(H) + 4 * H > cross_bytes(T) ? union_part(H) + 4 * H : cross_bytes(T);
+}
 constexpr int SCAN_THREADS = 1024;
 
 // longest-edge kernel: persistent warps, each with a two-stage ring of

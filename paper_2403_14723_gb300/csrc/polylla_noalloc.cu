@@ -37,7 +37,7 @@ constexpr size_t OFF_GROUP_PRE = OFF_GROUPS + up256(8 * (size_t)(NA_MAX_TILES / 
 constexpr size_t OFF_REC = OFF_GROUP_PRE + up256(8 * (size_t)(NA_MAX_TILES / SCAN_THREADS + 1));
 constexpr size_t OFF_WTOT = OFF_REC + up256(4 * (size_t)NA_MAX_T);
 constexpr size_t OFF_POOL = OFF_WTOT + up256(8 * (size_t)out_warp_count(NA_MAX_T));
-constexpr size_t OFF_CTRL = OFF_POOL + up256(64 * (size_t)(cross_own_count(NA_MAX_T) + cross_more_count(NA_MAX_T)));
+constexpr size_t OFF_CTRL = OFF_POOL + up256((size_t)cross_bytes(NA_MAX_T));
 constexpr size_t NA_BYTES = OFF_CTRL + up256(sizeof(DevCtrl));
 
 constexpr int kMaxDevices = 64;

@@ -103,13 +103,15 @@ struct Slot {
 // metadata), following the allocations of serve_reserve and the arena.
 int64_t slot_bytes(int64_t n, int64_t V, int64_t T, int64_t H) {
     const int64_t arena = 16 * V + 16 * H;
-    const int64_t uni = 16 * H + 20 * (n + 1) + 4 * seg_count(T);
+    // union_block is at most 16 KiB above its two arrays: 64 (T/8 + 256 + T/32 + T/8) - 24 T
+    // under 2,048 triangles, 58 T under 256
+    const int64_t uni = 16 * H + 16384 + 20 * (n + 1) + 4 * seg_count(T);
     const int64_t meta = 16 * n + 4 * (T + n + 1);
     const int64_t Tpad = (T + 15) / 16 * 16;
     const int64_t tiles = (T + OUT_TILE_MIN - 1) / OUT_TILE_MIN;
     const int64_t work = 2 * Tpad + 8 * V + 16 * tiles + 16 * (tiles / SCAN_THREADS + 1) +
                          4 * T + 8 * out_warp_count(T) +
-                         64 * (cross_own_count(T) + cross_more_count(T)) + 4 * T + 4 * (T + 1) + 24 * T + 256;
+                         4 * T + 4 * (T + 1) + 24 * T + 256;
     const int64_t lepp = 16 * ((T + 1023) / 1024 + 1) + 8;  // path-scan totals of the Lepp primitive
     return arena + uni + meta + work + lepp + 64 * 256;      // + small allocations and their rounding
 }
