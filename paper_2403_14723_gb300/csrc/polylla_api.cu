@@ -569,7 +569,10 @@ static int device_status(const DevCtrl &h) {
 }
 
 static int read_ctrl(polylla_ctx *c, cudaStream_t s) {
-    CK(launch_ctrl_out(c->w, c->h_ctrl, s));
+    // a kernel goes to streams of the current device only, a copy to any device's
+    int device = -1;
+    if (cudaGetDevice(&device) == cudaSuccess && device == c->device) CK(launch_ctrl_out(c->w, c->h_ctrl, s));
+    else CK(cudaMemcpyAsync(c->h_ctrl, c->w.ctrl, sizeof(DevCtrl), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     return POLYLLA_OK;
 }
