@@ -163,7 +163,15 @@ extern "C" int polylla_generate_noalloc(const polylla_mesh *mesh, int32_t *seeds
         launch_tile_scan(m, w, s, true);
         launch_poly_list(m, w, s, true);
     }
-    launch_kernel(k_noalloc_status, 1, 32, 0, s, true, static_cast<const DevCtrl *>(w.ctrl), status3);
+    // a kernel's stores need the words aligned, copies take any address
+    if (((uintptr_t)status3 & 3u) == 0) {
+        launch_kernel(k_noalloc_status, 1, 32, 0, s, true, static_cast<const DevCtrl *>(w.ctrl), status3);
+    } else if (cudaMemcpyAsync(status3, &w.ctrl->n_polygons, 2 * sizeof(int32_t), cudaMemcpyDeviceToDevice, s) !=
+                   cudaSuccess ||
+               cudaMemcpyAsync(reinterpret_cast<char *>(status3) + 8, &w.ctrl->error, sizeof(int32_t),
+                               cudaMemcpyDeviceToDevice, s) != cudaSuccess) {
+        return POLYLLA_ERR_CUDA;
+    }
     if (cudaGetLastError() != cudaSuccess) return POLYLLA_ERR_CUDA;
     return POLYLLA_OK;
 }
