@@ -54,11 +54,11 @@ void launch_validate(const MeshView &m, int32_t *bad, cudaStream_t s) {
 // Stage 1 on a mesh: longest_of (longest_edge.cuh) for every triangle.
 // ===========================================================================
 
-// Bound by latency and issue together (grid 2048 under ncu: 50.9 us, issue 61 %,
-// 32 warps per SM, DRAM 45 %, float64 pipe 31 %): whole generate of the 4096 grid
-// 1,121 -> 1,108 us with one bound for three edges, 1,076 -> 1,058 with the twins
-// read for ties only; 5 or 6 CTAs per SM (fewer registers) and the next set's
-// coordinates in flight during a label gained nothing.
+// Bound by latency and issue together (grid 2048 under ncu: 47 us, issue 62 %,
+// 28 warps per SM, 55 % of the measured copy rate, float64 pipe 34 %): whole
+// generate of the 4096 grid 1,121 -> 1,108 us with one bound for three edges,
+// 1,076 -> 1,058 with the twins read for ties only; 5 or 6 CTAs per SM (fewer
+// registers) and the next set's coordinates in flight during a label gained nothing.
 // Persistent warps walk tiles of 32 PER triangles.  Each warp owns a
 // two-stage shared-memory ring: lane 0 bulk-copies (TMA engine,
 // cp.async.bulk + mbarrier) the origin triples of the warp's next tile while
@@ -593,8 +593,8 @@ __global__ void __launch_bounds__(NT, 2048 / NT / IPT) k_label_relink(MeshView m
 // the walk-start mark.
 // Bound by instruction issue together with the latency of its chains of loads
 // (twin, label, twin, label): on the 2048 grid 93 M warp instructions at 3.1 a
-// cycle, 64 warps per SM; with 48 (40 registers) 0.428 ms on the 4096 grid, with
-// 40 0.520 ms, against 0.376 ms here and 0.387 ms with block barriers and a mark
+// cycle, 57 of 64 warps per SM; with at most 48 (40 registers) 0.428 ms on the 4096
+// grid, with 40 0.520 ms, against 0.376 ms here and 0.387 ms with block barriers and a mark
 // test for every half-edge.  Loads without branches (clamped indices past the
 // border) measured 0.407 ms.
 // ===========================================================================

@@ -22,9 +22,10 @@
 //   k_poly_list   gives every lane one word, so one polygon, places the
 //                 polygons by a warp scan of the lengths and lists them through
 //                 a staging buffer that goes out with coalesced stores.
-// Both are bound by instruction issue before memory: on the 2048 grid (8.4 M
-// triangles) the count issues 37.7 M warp instructions at 2.7 a cycle and moves
-// 36 % of the HBM peak, the listing 51 M at 2.4 and 64 %.  Against a lane per 4
+// The count is bound by instruction issue and latency, the listing by its bytes: on
+// the 2048 grid (8.4 M triangles, under ncu) the count issues 35.1 M warp
+// instructions at 2.5 a cycle and moves 140 MB in 49 us, 43 % of the measured copy
+// rate (6,696 GB/s), the listing 51.3 M at 2.4 and 358 MB in 72 us, 74 %.  Against a lane per 4
 // triangles that walked and listed whatever minima it held, each polygon that
 // left the tile stalling its lane's warp once in either kernel: count 0.168 ->
 // 0.172 ms, listing 0.395 -> 0.267 ms on the 4096 grid; 51 -> 33 and 49 -> 14 us

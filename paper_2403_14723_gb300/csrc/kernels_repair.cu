@@ -1,6 +1,6 @@
 // Repair-phase kernels (stage 5a): the chords of the barrier tips join the
-// frontier, and the links around their endpoints are redone.  Both run over the (short) tip list with a
-// persistent grid-stride loop, so a mesh without tips costs two tiny
+// frontier, and the links around their endpoints are redone.  Both run over the
+// (short) tip list in a grid-stride loop, so a mesh without tips costs two tiny
 // launches.
 #include "polylla_internal.cuh"
 

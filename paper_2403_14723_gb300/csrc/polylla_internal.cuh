@@ -177,7 +177,9 @@ constexpr int MBAR_WAIT_LIMIT = 1 << 22;
 // Every thread waits before it touches global memory, so a kernel has ended only
 // after all kernels before it; without a chained launch both are no-ops.  A pass of
 // 4 k triangles 87.8 -> 76.6 us, of 2 M 155.7 -> 146.6, of the 4096 grid 1,116 ->
-// 1,110.
+// 1,110.  The waiting blocks do not hold up another stream's short kernels: requests
+// of 20 k triangles in the server's lane beside back-to-back generates of 8.4 M took
+// 0.270 ms (p99 0.298) with the chain, 0.280 (0.359) without it.
 // A chained kernel is resident while the kernels before it still write, so only
 // what no kernel of its chain writes may be read through the read-only path
 // (__ldg, const __restrict__): the caller's mesh arrays (coords, origin, twin) and
